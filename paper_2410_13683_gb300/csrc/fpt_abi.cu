@@ -1032,7 +1032,8 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
     int occ = em_occupancy(var, block, smem_bytes);
     if (occ < 1) return fail(ctx, FPT_E_CUDA, "stepper does not fit on an SM with this shape");
     const int bps = ctx->launch.blocks_per_sm ? std::min(ctx->launch.blocks_per_sm, occ) : occ;
-    const int grid = std::max(1, bps * ctx->sm_count);
+    // no more blocks than chunks of 32 trajectories: a block's first warp takes a chunk each
+    const int grid = (int)std::max<long long>(1, std::min<long long>((long long)bps * ctx->sm_count, (total + 31) / 32));
     // the learned proposal is re-evaluated at every refill point
     const int check_steps = mlp ? runs[mlp_run].mlp_segment : ctx->launch.check_steps;
 
@@ -1063,6 +1064,8 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
         }
     }
     p.groups_per_check = check_steps / 4;
+    p.tail_intervals = std::max(1, 128 / check_steps);
+    p.sm_count = ctx->sm_count;
     p.mlp_run = mlp ? mlp_run : 0;
     p.records = ctx->d_records;
     p.rec_cursor = ctx->d_rec_cursor;

@@ -147,8 +147,7 @@ struct Lane {                // per-thread trajectory state and its constants
     float x, x_c;            // shifted field phi - phi_end as a Kahan pair: x - x_c
     float p, p_c;            // momentum; p_c compensates it (Kahan) in the variants with pi-noise
     float lw_hi, lw_lo;      // ln w as a Kahan pair
-    float lw_grp;            // increments of the current 4-step group, added to the pair per group
-    int n;
+    int grp;                 // steps taken / 4 (a live lane's count is a multiple of 4 between groups)
     int nmax;
     uint32_t traj, run_id;
     float cb, half_cb2, dN, sqrt_dN;
@@ -164,7 +163,7 @@ struct Lane {                // per-thread trajectory state and its constants
     bool nidx;               // noise table indexed by the step count
     int win_lo, win_hi;      // noise window in steps (nidx)
     int run;                 // index of the lane's run in the launch
-    long long unit;
+    uint32_t unit;           // launch unit (a launch has at most 2^32)
 };
 
 struct SegRec {              // open segment of the record variant
@@ -186,7 +185,7 @@ __device__ __forceinline__ void lane_load(Lane &L, long long unit, const RunSm *
     const RunSm &r = s_run[lo];
     const ModelDev &m = s_model[r.model];
     L.run = lo;
-    L.unit = unit;
+    L.unit = (uint32_t)unit;
     L.traj = (uint32_t)(r.traj_offset + (unit - r.unit_begin));
     L.run_id = r.run_id;
     L.cb = r.cb;
@@ -222,8 +221,7 @@ __device__ __forceinline__ void lane_load(Lane &L, long long unit, const RunSm *
     L.p_c = 0.0f;
     L.lw_hi = 0.0f;
     L.lw_lo = 0.0f;
-    L.lw_grp = 0.0f;
-    L.n = 0;
+    L.grp = 0;
 }
 
 // Table entry and interpolation weight at the lane's field. The 1-D tables
@@ -235,11 +233,11 @@ __device__ __forceinline__ void lane_load(Lane &L, long long unit, const RunSm *
 // zero slope, so every reachable k (0 .. M-1) is a valid entry.
 template <bool SMEM, bool NIDX = false>
 __device__ __forceinline__ float4 table_at(const Lane &L, const float4 *__restrict__ tab, float &f,
-                                           const ModelDev &M0)
+                                           const ModelDev &M0, int n = 0)
 {
     const float kMagic = 12582912.0f;                        // 1.5 * 2^23
     // N-indexed tables: coordinate from the exact step count (n < 2^24 is exact in FP32)
-    const float coord = (NIDX && L.nidx) ? __int2float_rn(L.n) : L.x;
+    const float coord = (NIDX && L.nidx) ? __int2float_rn(n) : L.x;
     float u = fmaf(coord, SMEM ? M0.u_scale : L.u_scale, SMEM ? M0.u_shift : L.u_shift);
     u = fminf(fmaxf(u, -0.5f), SMEM ? M0.u_umax : L.u_max);
     const float t = u + kMagic;
@@ -318,23 +316,23 @@ __device__ __forceinline__ float hh_dN(const Lane &L, const ModelDev &M0)
     return fmaf(h * L.p, L.p, m3);
 }
 
-// One Euler-Maruyama step of Eq. (4.7) with bias amplitude L.cb / sqrt(dN).
-// The field increment (drift + bias + noise) is formed first and added to the
-// compensated field pair: a plain FP32 field would add the same drift
-// increment to a value on its own grid every step, a rounding error with a
-// fixed sign. Returns true when the trajectory has finished (passage or cap).
+// One Euler-Maruyama step of Eq. (4.7) with bias amplitude L.cb / sqrt(dN),
+// step number n. The field increment (drift + bias + noise) is formed first and
+// added to the compensated field pair: a plain FP32 field would add the same
+// drift increment to a value on its own grid every step, a rounding error with
+// a fixed sign. lw: ln w increments of the current group.
 template <bool WEIGHTED, bool SMEM, bool NIDX = false, bool DTAB = false>
-__device__ __forceinline__ bool em_step(Lane &L, float z, const float4 *__restrict__ tab,
+__device__ __forceinline__ void em_step(Lane &L, int n, float z, float &lw, const float4 *__restrict__ tab,
                                         const ModelDev *s_model, const ModelDev &M0)
 {
     // noise table: linear interpolation in x (or in time), end values held outside
     float f;
-    const float4 e = table_at<SMEM, NIDX>(L, tab, f, M0);
+    const float4 e = table_at<SMEM, NIDX>(L, tab, f, M0, n);
     const float dN = SMEM ? M0.dN : L.dN;
     float S = fmaf(f, e.y, e.x);               // S_phiphi sqrt(dN)
     float T = fmaf(f, e.w, e.z);               // tan(theta_n) S_phiphi sqrt(dN)
     float cb = L.cb, half_cb2 = L.half_cb2;
-    if (outside_window<NIDX>(L, L.n)) {
+    if (outside_window<NIDX>(L, n)) {
         // outside the noise window the step is classical: no noise, no bias, no weight
         S = 0.0f;
         T = 0.0f;
@@ -352,23 +350,22 @@ __device__ __forceinline__ bool em_step(Lane &L, float z, const float4 *__restri
     } else {
         L.p = fmaf(T, zb, fmaf(hdN, L.p + vpv, L.p));
     }
-    if (WEIGHTED) L.lw_grp -= fmaf(cb, z, half_cb2);   // the step's ln w increment (see group_lw)
+    if (WEIGHTED) lw -= fmaf(cb, z, half_cb2);          // the step's ln w increment (see group_lw)
     kahan_add(L.x, L.x_c, dx);
-    ++L.n;
-    return passed(L) | (L.n >= (SMEM ? M0.max_steps : L.nmax));
 }
 
 // ln w increments of the first k + 1 steps of a group that starts at step
-// n0, summed as em_step sums them (same operands, same order).
-template <bool NIDX>
-__device__ __forceinline__ float group_lw(const Lane &L, const float (&z)[4], int n0, int k)
+// n0, summed as the steps sum them (same operands, same order).
+template <bool NIDX, bool RANK2>
+__device__ __forceinline__ float group_lw(const Lane &L, const float *z, int n0, int k)
 {
     float lw = 0.0f;
 #pragma unroll
     for (int s = 0; s < 4; ++s) {
         if (s > k) break;
         const bool off = outside_window<NIDX>(L, n0 + s);
-        lw -= fmaf(off ? 0.0f : L.cb, z[s], off ? 0.0f : L.half_cb2);
+        const float cb = off ? 0.0f : L.cb, half_cb2 = off ? 0.0f : L.half_cb2;
+        lw -= RANK2 ? fmaf(cb, z[2 * s], fmaf(L.cb_b, z[2 * s + 1], half_cb2)) : fmaf(cb, z[s], half_cb2);
     }
     return lw;
 }
@@ -394,7 +391,7 @@ __device__ __forceinline__ void mlp_segment_start(Lane &L, bool live, SegRec &sg
         in0 = ((pr.mlp_flags & FPT_MLP_LOG_X) ? __logf(fmaxf(xv, pr.x_floor)) : xv);
         in0 = (in0 - pr.shift[0]) * pr.scale[0];
         in1 = (L.p - pr.shift[1]) * pr.scale[1];
-        in2 = ((float)L.n * dN - pr.shift[2]) * pr.scale[2];
+        in2 = ((float)(4 * L.grp) * dN - pr.shift[2]) * pr.scale[2];
         float f;
         const float4 e = table_at<SMEM>(L, tab, f, M0);
         const float S = fmaf(f, e.y, e.x), T = fmaf(f, e.w, e.z);
@@ -410,7 +407,7 @@ __device__ __forceinline__ void mlp_segment_start(Lane &L, bool live, SegRec &sg
         if (REC) {
             sg.in0 = in0; sg.in1 = in1; sg.in2 = in2; sg.tan_t = tan_t; sg.raw = raw;
             sg.sum_xi = 0.0f;
-            sg.n0 = L.n;
+            sg.n0 = 4 * L.grp;
             sg.open = true;
         }
     }
@@ -439,7 +436,7 @@ __device__ __forceinline__ void mlp_segment_start_multi(Lane &L, bool live, SegR
             in0 = ((pr.mlp_flags & FPT_MLP_LOG_X) ? __logf(fmaxf(xv, pr.x_floor)) : xv);
             in0 = (in0 - pr.shift[0]) * pr.scale[0];
             in1 = (L.p - pr.shift[1]) * pr.scale[1];
-            in2 = ((float)L.n * dN - pr.shift[2]) * pr.scale[2];
+            in2 = ((float)(4 * L.grp) * dN - pr.shift[2]) * pr.scale[2];
             float f;
             const float4 e = table_at<SMEM>(L, tab, f, M0);
             const float S = fmaf(f, e.y, e.x), T = fmaf(f, e.w, e.z);
@@ -457,7 +454,7 @@ __device__ __forceinline__ void mlp_segment_start_multi(Lane &L, bool live, SegR
             if (REC) {
                 sg.in0 = in0; sg.in1 = in1; sg.in2 = in2; sg.tan_t = tan_t; sg.raw = raw;
                 sg.sum_xi = 0.0f;
-                sg.n0 = L.n;
+                sg.n0 = 4 * L.grp;
                 sg.open = true;
             }
         }
@@ -525,48 +522,156 @@ __device__ __forceinline__ void stage_launch(const EmParams &P, float4 *s_tab, R
     __syncthreads();
 }
 
-// Refill point: write the warp's finished trajectories and fetch new units
-// with one warp-aggregated atomic on the work cursor.
-__device__ __forceinline__ void refill_point(const EmParams &P, Lane &L, bool &active, bool &done,
-                                             const RunSm *s_run, const ModelDev *s_model)
+// A trajectory that has ended after n steps: its results, written once.
+__device__ __forceinline__ void finish(const EmParams &P, const Lane &L, int n, bool pas)
 {
-    const unsigned FULL = 0xffffffffu;
-    const unsigned lane = threadIdx.x & 31u;
-    const bool fin_me = active && done;
-    const unsigned fin = __ballot_sync(FULL, fin_me);
-    if (!fin) return;
-    if (fin_me) {
-        const bool pas = passed(L);
-        CHECK_INDEX(L.unit, P.total_units, kCheckUnit);
-        P.nsteps[L.unit] = L.n;
-        P.logw[L.unit] = (double)L.lw_hi - (double)L.lw_lo;     // the pair holds hi - lo
-        P.status[L.unit] = pas ? (uint8_t)FPT_TRAJ_PASSED : (uint8_t)FPT_TRAJ_CAPPED;
-        if (!pas) atomicAdd(P.flags + 1, 1);
-    }
-    unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(P.cursor, (unsigned long long)__popc(fin));
-    base = __shfl_sync(FULL, base, 0);
-    if (fin_me) {
-        const long long unit = (long long)(base + __popc(fin & ((1u << lane) - 1u)));
-        done = false;
-        active = unit < P.total_units;
-        if (active) lane_load(L, unit, s_run, s_model, P.n_runs);
-    }
+    long long u = L.unit;
+    CHECK_INDEX(u, P.total_units, kCheckUnit);
+    P.nsteps[u] = n;
+    P.logw[u] = (double)L.lw_hi - (double)L.lw_lo;     // the pair holds hi - lo
+    P.status[u] = pas ? (uint8_t)FPT_TRAJ_PASSED : (uint8_t)FPT_TRAJ_CAPPED;
+    if (!pas) atomicAdd(P.flags + kFlagCapped, 1);
 }
 
-// First units of a warp.
-__device__ __forceinline__ void first_units(const EmParams &P, Lane &L, bool &active,
-                                            const RunSm *s_run, const ModelDev *s_model)
+// First units of a warp: chunk c of 32 units goes to block c mod grid, so that a
+// launch with fewer chunks than resident warps loads every SM alike (taken from
+// the cursor instead, the first blocks to start took 16 chunks each: 16,384
+// paths ran on a quarter of the SMs, 2.26 ms a launch against 0.60 ms; eight
+// runs of 20,011 paths, most of them capped at 2^18 steps, 125 -> 74 ms). Within a
+// block the chunks go to warps in the order of warp_at(), rotated for the
+// blocks that share an SM, so that their first warps sit on different
+// sub-partitions.
+__device__ __forceinline__ int block_rotation(const EmParams &P)
+{
+    return (int)((blockIdx.x / (unsigned)P.sm_count) % (blockDim.x >> 5));
+}
+
+__device__ __forceinline__ bool first_units(const EmParams &P, Lane &L, const RunSm *s_run,
+                                            const ModelDev *s_model)
+{
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int pos = (warp + nw - block_rotation(P)) % nw;
+    const long long unit = ((long long)pos * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31u);
+    // lanes without a trajectory step along harmlessly on zeros: every table index is clamped
+    L = Lane{};
+    L.M = 1;
+    if (unit >= P.total_units) return false;
+    lane_load(L, unit, s_run, s_model, P.n_runs);
+    return true;
+}
+
+// Refill point: lanes without a trajectory fetch new units with one
+// warp-aggregated atomic on the work cursor (units past the launch's first
+// ones). Returns true when a lane was loaded; s_dry is set once the cursor has
+// run past the last unit.
+__device__ __forceinline__ bool refill_point(const EmParams &P, Lane &L, bool &live, const RunSm *s_run,
+                                             const ModelDev *s_model, int *s_dry)
 {
     const unsigned FULL = 0xffffffffu;
     const unsigned lane = threadIdx.x & 31u;
+    const unsigned idle = __ballot_sync(FULL, !live);
+    if (!idle) return false;
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(P.cursor, 32ull);
-    base = __shfl_sync(FULL, base, 0);
-    const long long unit = (long long)(base + lane);
-    active = unit < P.total_units;
-    if (active) lane_load(L, unit, s_run, s_model, P.n_runs);
-    else L.n = 0, L.traj = 0, L.run_id = 0, L.mlp = false, L.nidx = false, L.run = 0;
+    if (lane == 0) base = atomicAdd(P.cursor, (unsigned long long)__popc(idle));
+    base = __shfl_sync(FULL, base, 0) + (unsigned long long)gridDim.x * blockDim.x;
+    if ((long long)base + __popc(idle) > P.total_units && lane == 0) *(volatile int *)s_dry = 1;
+    bool got = false;
+    if (!live) {
+        const long long unit = (long long)(base + __popc(idle & ((1u << lane) - 1u)));
+        if (unit < P.total_units) {
+            lane_load(L, unit, s_run, s_model, P.n_runs);
+            live = got = true;
+        }
+    }
+    return __any_sync(FULL, got);
+}
+
+// ---------------------------------------------------------------------------
+// The launch's tail: compaction of the block's live lanes
+// ---------------------------------------------------------------------------
+// Path lengths are heavy-tailed, so once the work cursor is dry the warps keep
+// one or two live lanes each for most of a launch, at the price of full ones.
+// From then on (tail mode) the warps of a block meet every tail_intervals
+// intervals (128 steps) and the live lanes of the last warps move into free
+// lanes of the first ones, through a small pool in shared memory, whenever that
+// empties a warp. A lane's state is eight words; everything else is loaded
+// from its run and model again. A lane moves between intervals, where no group
+// and no held-alpha segment is open, so results do not depend on it. Measured
+// with the straight-line groups below: 2^18 learned paths (median 8,902 steps,
+// longest 262,144) 78 -> 34 ms, where the longest path's step took 324 ns
+// among 24 sparse warps per SM; 64 models x 8,192 paths 76 -> 32 ms.
+constexpr int kPoolLanes = 128;          // lanes one compaction can move (4 KB of shared memory)
+constexpr int kMaxWarps = 16;
+
+struct TailSm {
+    float4 pool[2 * kPoolLanes];
+    int count[2][kMaxWarps];             // live lanes per warp, double-buffered by round
+    int dry;
+};
+
+__device__ __forceinline__ int warp_at(int pos, int rot, int nw)
+{
+    const int w = pos + rot;
+    return w >= nw ? w - nw : w;
+}
+
+// One meeting of the block's warps. Returns -1 when the block has no live lane
+// left (or must stop), else 1 when this warp's lanes changed, 0 when not.
+__device__ __forceinline__ int tail_meeting(const EmParams &P, Lane &L, bool &live, bool stop, int round,
+                                            TailSm &T, const RunSm *s_run, const ModelDev *s_model)
+{
+    const unsigned FULL = 0xffffffffu;
+    const unsigned lane = threadIdx.x & 31u;
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, rot = block_rotation(P);
+    const unsigned mask = __ballot_sync(FULL, live);
+    int *cnt = T.count[round & 1];
+    if (lane == 0) cnt[warp] = __popc(mask);
+    if (__syncthreads_or(stop)) return -1;
+    int total = 0, used = 0;
+    for (int j = 0; j < nw; ++j) {
+        total += cnt[j];
+        used += cnt[j] > 0;
+    }
+    if (!total) return -1;
+    // keep the first `keep` positions; the later ones' lanes must fit the pool
+    int keep = nw, moved = 0;
+    const int need = (total + 31) >> 5;
+    if (need < used) {
+        while (keep > need && moved + cnt[warp_at(keep - 1, rot, nw)] <= kPoolLanes)
+            moved += cnt[warp_at(--keep, rot, nw)];
+    }
+    if (!moved) return 0;
+    // donors in order of position fill the pool, free lanes in the same order empty it
+    int before = 0, pos = 0;
+    for (int j = 0; j < nw; ++j) {
+        const int w = warp_at(j, rot, nw);
+        if (w == warp) { pos = j; break; }
+        if (j < keep) before += 32 - cnt[w];
+    }
+    const bool donor = pos >= keep;
+    if (donor) {
+        before = 0;
+        for (int j = keep; j < pos; ++j) before += cnt[warp_at(j, rot, nw)];
+        if (live) {
+            const int e = before + __popc(mask & ((1u << lane) - 1u));
+            T.pool[2 * e] = make_float4(L.x, L.x_c, L.p, L.p_c);
+            T.pool[2 * e + 1] = make_float4(L.lw_hi, L.lw_lo, __int_as_float(L.grp), __uint_as_float(L.unit));
+            live = false;
+        }
+    }
+    __syncthreads();
+    if (donor) return 0;
+    const int e = before + __popc(~mask & ((1u << lane) - 1u));
+    const bool take = !live && e < moved;
+    if (take) {
+        const float4 a = T.pool[2 * e], b = T.pool[2 * e + 1];
+        lane_load(L, (long long)__float_as_uint(b.w), s_run, s_model, P.n_runs);
+        L.x = a.x; L.x_c = a.y; L.p = a.z; L.p_c = a.w;
+        L.lw_hi = b.x; L.lw_lo = b.y;
+        L.grp = __float_as_int(b.z);
+        live = true;
+    }
+    return __any_sync(FULL, take) ? 1 : 0;
 }
 
 // Deadline: true when the launch should stop (lane 0 reads the device clock).
@@ -580,151 +685,36 @@ __device__ __forceinline__ bool past_deadline(const EmParams &P, unsigned long l
     return __shfl_sync(0xffffffffu, stop, 0) != 0;
 }
 
-// Close the warp's open segments at a refill point: record r holds
-// q0 = (inputs, slot 3) and q1 = (slot 4, slot 5, unit, first step of the
-// segment), appended with one warp-aggregated atomic on the record cursor;
-// records past the buffer raise flag 3 instead of being written.
-__device__ __forceinline__ void write_records(const EmParams &P, const Lane &L, SegRec &sg, bool active,
-                                              float4 q0, float s4, float s5)
+// Segment record idx: q0 = (inputs, tan theta_n), q1 = (raw alpha, sum xi, unit,
+// first step); full-rank noise: q0 = (inputs, sum xi_2), q1 = (0, sum xi_1, unit,
+// first step). Records past the buffer raise a flag instead of being written.
+template <bool RANK2>
+__device__ __forceinline__ void put_record(const EmParams &P, const Lane &L, const SegRec &sg, long long idx)
+{
+    if (idx < P.rec_cap) {
+        float4 *q = reinterpret_cast<float4 *>(P.records + 8 * idx);
+        q[0] = make_float4(sg.in0, sg.in1, sg.in2, RANK2 ? sg.sum_xi2 : sg.tan_t);
+        q[1] = make_float4(RANK2 ? 0.0f : sg.raw, sg.sum_xi, __uint_as_float(L.unit), __int_as_float(sg.n0));
+    } else {
+        atomicExch(P.flags + kFlagRecOverflow, 1);
+    }
+}
+
+// Close the warp's open segments at a refill point, appended with one
+// warp-aggregated atomic on the record cursor.
+template <bool RANK2>
+__device__ __forceinline__ void write_records(const EmParams &P, const Lane &L, SegRec &sg)
 {
     const unsigned FULL = 0xffffffffu;
     const unsigned lane = threadIdx.x & 31u;
-    const bool wr = active && sg.open;
-    const unsigned m = __ballot_sync(FULL, wr);
+    const unsigned m = __ballot_sync(FULL, sg.open);
     if (m) {
         unsigned long long base = 0;
         if (lane == 0) base = atomicAdd(P.rec_cursor, (unsigned long long)__popc(m));
         base = __shfl_sync(FULL, base, 0);
-        if (wr) {
-            const long long idx = (long long)(base + __popc(m & ((1u << lane) - 1u)));
-            if (idx < P.rec_cap) {
-                float4 *q = reinterpret_cast<float4 *>(P.records + 8 * idx);
-                q[0] = q0;
-                q[1] = make_float4(s4, s5, __uint_as_float((uint32_t)L.unit), __int_as_float(sg.n0));
-            } else {
-                atomicExch(P.flags + 3, 1);
-            }
-        }
+        if (sg.open) put_record<RANK2>(P, L, sg, (long long)(base + __popc(m & ((1u << lane) - 1u))));
     }
     sg.open = false;
-}
-
-// Register budgets: the plain stepper keeps three 512-thread blocks per SM
-// (48 warps, 40 registers); the noise-window and bump steppers two 512-thread
-// blocks; the learned-proposal steppers at most 384 threads per block and two
-// blocks, 80 registers: the network's fragments fit without spilling (a
-// 64-register build ran 512-thread blocks but executed ~7% more instructions
-// per step, and the autotuner chose 384 threads for it anyway).
-template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET = false>
-__global__ void __launch_bounds__(MLP ? kMlpMaxBlock : 512, (MLP || NIDX || DTAB) ? 2 : 3)
-    em_kernel(const EmParams P)
-{
-    extern __shared__ __align__(16) float4 s_tab[];
-    __shared__ unsigned long long s_t0;
-
-    // single-network MLP variants: the proposal's fragment blob follows the
-    // table in shared memory; then the run constants and model descriptors
-    const int tab_entries = SMEM ? P.smem_table_points : 0;
-    uint2 *s_tiles = reinterpret_cast<uint2 *>(s_tab + tab_entries);
-    float *s_bias = reinterpret_cast<float *>(s_tiles + kMlpTiles * 32);
-    RunSm *s_run = smem_runs(s_tab, tab_entries, MLP && !MNET);
-    ModelDev *s_model = smem_models(s_run, P.n_runs);
-    const RunDev &prun = P.runs[MLP ? P.mlp_run : 0];
-    stage_launch<SMEM, MLP && !MNET>(P, s_tab, s_run, s_model, s_t0, s_tiles);
-
-    const float4 *tab = SMEM ? s_tab : P.tables;
-    const unsigned FULL = 0xffffffffu;
-
-    Lane L;
-    SegRec sg;
-    sg.open = false;
-    bool active = false, done = false;
-    first_units(P, L, active, s_run, s_model);
-
-    for (;;) {
-        if (MLP && __any_sync(FULL, active && L.mlp)) {
-            if (MNET) mlp_segment_start_multi<SMEM, REC>(L, active && L.mlp, sg, tab, P.runs, P.m0);
-            else mlp_segment_start<SMEM, REC>(L, active && L.mlp, sg, tab, s_tiles, s_bias, prun, P.m0);
-        }
-
-        // Speculative groups (single-model launches): when every lane of the
-        // warp is live and the whole interval stays below the cap, the four steps
-        // of a group run without the per-step branch, each lane noting after
-        // which steps its field was at or below the end surface. A lane that
-        // passed at step k of the group then takes the state the guarded path
-        // would have left: k + 1 steps counted, the ln w increments of those
-        // steps summed again from the same operands, its field marked passed
-        // (the later steps' field and momentum are discarded: the trajectory has
-        // ended, and only its step count, weight and status are kept), and the
-        // warp's remaining groups of the interval run guarded. Results do not
-        // depend on which path ran.
-        bool spec = SMEM && __all_sync(FULL, active && !done &&
-                                                 L.n + 4 * P.groups_per_check < P.m0.max_steps);
-        for (int g = 0; g < P.groups_per_check; ++g) {
-            const uint4 r = philox4x32_10(make_uint4((uint32_t)L.n >> 2, L.traj, L.run_id, 0u), P.rk);
-            float z[4];
-            box_muller(r.x, r.y, z[0], z[1]);
-            box_muller(r.z, r.w, z[2], z[3]);
-            if (spec) {
-                const float sx0 = REC ? sg.sum_xi : 0.0f;
-                bool h[4];
-#pragma unroll
-                for (int s = 0; s < 4; ++s) {
-                    if (REC) sg.sum_xi = __fadd_rn(sg.sum_xi, z[s]);
-                    em_step<WEIGHTED, SMEM, NIDX, DTAB>(L, z[s], tab, s_model, P.m0);
-                    h[s] = passed(L);
-                }
-                const bool hit = h[0] | h[1] | h[2] | h[3];
-                if (__any_sync(FULL, hit)) spec = false;
-                if (hit) {
-                    const int k = h[0] ? 0 : h[1] ? 1 : h[2] ? 2 : 3;
-                    const int n0 = L.n - 4;
-                    // the group's normals again (not kept live through the steps)
-                    const uint4 q = philox4x32_10(make_uint4((uint32_t)n0 >> 2, L.traj, L.run_id, 0u), P.rk);
-                    float zz[4];
-                    box_muller(q.x, q.y, zz[0], zz[1]);
-                    box_muller(q.z, q.w, zz[2], zz[3]);
-                    L.n = n0 + k + 1;
-                    if (WEIGHTED) L.lw_grp = group_lw<NIDX>(L, zz, n0, k);
-                    if (REC) {
-                        float sx = sx0;
-#pragma unroll
-                        for (int s = 0; s < 4; ++s)
-                            if (s <= k) sx = __fadd_rn(sx, zz[s]);
-                        sg.sum_xi = sx;
-                    }
-                    L.x = -1.0f;
-                    L.x_c = 0.0f;
-                    done = true;
-                }
-            } else {
-#pragma unroll
-                for (int s = 0; s < 4; ++s)
-                    if (active && !done) {
-                        if (REC) sg.sum_xi = __fadd_rn(sg.sum_xi, z[s]);
-                        done = em_step<WEIGHTED, SMEM, NIDX, DTAB>(L, z[s], tab, s_model, P.m0);
-                    }
-            }
-            // the group's weight increments (at most 4, so a plain FP32 sum) into the
-            // pair; a lane that took no step in the group adds nothing (re-adding zero
-            // would re-round the pair, and how often depends on the launch shape)
-            if (WEIGHTED && L.lw_grp != 0.0f) {
-                kahan_add(L.lw_hi, L.lw_lo, L.lw_grp);
-                L.lw_grp = 0.0f;
-            }
-        }
-
-        if (REC) {
-            // close the segments of this interval: (inputs, tan, raw alpha, sum xi, unit, steps)
-            write_records(P, L, sg, active, make_float4(sg.in0, sg.in1, sg.in2, sg.tan_t), sg.raw, sg.sum_xi);
-        }
-
-        // refill point: write finished trajectories, fetch new work
-        refill_point(P, L, active, done, s_run, s_model);
-        if (!__any_sync(FULL, active)) break;
-        // trajectories in flight keep the ABORTED status set before launch
-        if (P.budget_ns && past_deadline(P, s_t0)) break;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -756,7 +746,7 @@ __device__ __forceinline__ void table2_at(const Lane &L, const float4 *__restric
 }
 
 template <bool WEIGHTED, bool SMEM, bool DTAB>
-__device__ __forceinline__ bool em2_step(Lane &L, float z1, float z2, const float4 *__restrict__ tab,
+__device__ __forceinline__ void em2_step(Lane &L, float z1, float z2, float &lw, const float4 *__restrict__ tab,
                                          const ModelDev *s_model, const ModelDev &M0)
 {
     float a, b, c;                                       // S sqrt(dN), interpolated in x
@@ -769,10 +759,8 @@ __device__ __forceinline__ bool em2_step(Lane &L, float z1, float z2, const floa
     const float dx = fmaf(a, e1, fmaf(b, e2, L.p * dN));
     // full-rank noise drives pi directly: compensated momentum (see em_step)
     kahan_add(L.p, L.p_c, fmaf(b, e1, fmaf(c, e2, hdN * (L.p + vpv))));
-    if (WEIGHTED) L.lw_grp -= fmaf(L.cb, z1, fmaf(L.cb_b, z2, L.half_cb2));
+    if (WEIGHTED) lw -= fmaf(L.cb, z1, fmaf(L.cb_b, z2, L.half_cb2));
     kahan_add(L.x, L.x_c, dx);
-    ++L.n;
-    return passed(L) | (L.n >= (SMEM ? M0.max_steps : L.nmax));
 }
 
 // Learned proposal in 2-D: beta = (clamp(o1), clamp(o2)) at the segment start.
@@ -787,7 +775,7 @@ __device__ __forceinline__ void mlp2_segment_start(Lane &L, bool live, SegRec &s
         in0 = ((pr.mlp_flags & FPT_MLP_LOG_X) ? __logf(fmaxf(xv, pr.x_floor)) : xv);
         in0 = (in0 - pr.shift[0]) * pr.scale[0];
         in1 = (L.p - pr.shift[1]) * pr.scale[1];
-        in2 = ((float)L.n * dN - pr.shift[2]) * pr.scale[2];
+        in2 = ((float)(4 * L.grp) * dN - pr.shift[2]) * pr.scale[2];
     }
     float o1, o2;
     mlp_forward_warp(tiles, bias, in0, in1, in2, o1, o2);
@@ -801,121 +789,208 @@ __device__ __forceinline__ void mlp2_segment_start(Lane &L, bool live, SegRec &s
             sg.in0 = in0; sg.in1 = in1; sg.in2 = in2;
             sg.sum_xi = 0.0f;
             sg.sum_xi2 = 0.0f;
-            sg.n0 = L.n;
+            sg.n0 = 4 * L.grp;
             sg.open = true;
         }
     }
 }
 
-template <bool WEIGHTED, bool SMEM, bool MLP, bool DTAB, bool REC = false>
-__global__ void __launch_bounds__(MLP ? kMlpMaxBlock : 512, 2) em2_kernel(const EmParams P)
+// ---------------------------------------------------------------------------
+// The interval between two refill points
+// ---------------------------------------------------------------------------
+// One group of four steps of every lane, in either noise rank.
+template <bool WEIGHTED, bool SMEM, bool NIDX, bool DTAB, bool RANK2>
+__device__ __forceinline__ void any_step(Lane &L, int n, int s, const float *z, float &lw,
+                                         const float4 *__restrict__ tab, const ModelDev *s_model,
+                                         const ModelDev &M0)
+{
+    if (RANK2) em2_step<WEIGHTED, SMEM, DTAB>(L, z[2 * s], z[2 * s + 1], lw, tab, s_model, M0);
+    else em_step<WEIGHTED, SMEM, NIDX, DTAB>(L, n, z[s], lw, tab, s_model, M0);
+}
+
+// Normals of group grp: Philox block grp (1-D noise: one normal per step), blocks
+// 2 grp and 2 grp + 1 (full-rank noise: two per step).
+template <bool RANK2>
+__device__ __forceinline__ void group_normals(const EmParams &P, const Lane &L, int grp, float *z)
+{
+#pragma unroll
+    for (int h = 0; h < (RANK2 ? 2 : 1); ++h) {
+        const uint4 r = philox4x32_10(make_uint4((RANK2 ? 2u : 1u) * (uint32_t)grp + h, L.traj, L.run_id, 0u), P.rk);
+        box_muller(r.x, r.y, z[4 * h], z[4 * h + 1]);
+        box_muller(r.z, r.w, z[4 * h + 2], z[4 * h + 3]);
+    }
+}
+
+// Sums of normals over the first k + 1 steps of a group (record mode).
+template <bool RANK2>
+__device__ __forceinline__ void add_xi(SegRec &sg, const float *z, int k)
+{
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        if (s > k) break;
+        sg.sum_xi = __fadd_rn(sg.sum_xi, z[RANK2 ? 2 * s : s]);
+        if (RANK2) sg.sum_xi2 = __fadd_rn(sg.sum_xi2, z[2 * s + 1]);
+    }
+}
+
+// Every lane of the warp steps through the group, without a branch per step; a
+// lane notes after which steps its field was at or below the end surface. A
+// live lane that passed at step k ends there: its step count is 4 grp + k + 1,
+// its ln w and noise sums are formed from the increments of those k + 1 steps,
+// in the same order as the running sums, and its results are written at once.
+// What the lane computes after that (until it is refilled) is never read, and
+// every table index is clamped, so it stays in bounds. A warp with idle lanes
+// thus runs the same straight code as a full one.
+template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
+__device__ __forceinline__ void run_group(const EmParams &P, Lane &L, bool &live, SegRec &sg,
+                                          const float4 *__restrict__ tab, const ModelDev *s_model)
+{
+    float z[RANK2 ? 8 : 4];
+    group_normals<RANK2>(P, L, L.grp, z);
+    const int n0 = 4 * L.grp;
+    float lw = 0.0f;
+    bool h[4];
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        any_step<WEIGHTED, SMEM, NIDX, DTAB, RANK2>(L, n0 + s, s, z, lw, tab, s_model, P.m0);
+        h[s] = passed(L);
+    }
+    if (live && (h[0] | h[1] | h[2] | h[3])) {
+        const int k = h[0] ? 0 : h[1] ? 1 : h[2] ? 2 : 3;
+        if (WEIGHTED) {
+            const float lk = group_lw<NIDX, RANK2>(L, z, n0, k);
+            if (lk != 0.0f) kahan_add(L.lw_hi, L.lw_lo, lk);
+        }
+        finish(P, L, n0 + k + 1, true);
+        live = false;
+        if (REC && sg.open) {
+            add_xi<RANK2>(sg, z, k);
+            put_record<RANK2>(P, L, sg, (long long)atomicAdd(P.rec_cursor, 1ull));
+            sg.open = false;
+        }
+    }
+    if (REC) add_xi<RANK2>(sg, z, 3);
+    // the group's weight increments (at most 4, so a plain FP32 sum) into the pair;
+    // adding a zero sum would re-round the pair
+    if (WEIGHTED && lw != 0.0f) kahan_add(L.lw_hi, L.lw_lo, lw);
+    ++L.grp;
+}
+
+// The same with a branch per step, for the interval in which a lane of the warp
+// reaches the step cap inside a group.
+template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
+__device__ __forceinline__ void run_group_guarded(const EmParams &P, Lane &L, bool &live, SegRec &sg,
+                                                  const float4 *__restrict__ tab, const ModelDev *s_model)
+{
+    float z[RANK2 ? 8 : 4];
+    group_normals<RANK2>(P, L, L.grp, z);
+    const int nmax = SMEM ? P.m0.max_steps : L.nmax;
+    int n = 4 * L.grp;
+    float lw = 0.0f;
+    bool done = !live;
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+        if (!done) {
+            if (REC) {
+                sg.sum_xi = __fadd_rn(sg.sum_xi, z[RANK2 ? 2 * s : s]);
+                if (RANK2) sg.sum_xi2 = __fadd_rn(sg.sum_xi2, z[2 * s + 1]);
+            }
+            any_step<WEIGHTED, SMEM, NIDX, DTAB, RANK2>(L, n, s, z, lw, tab, s_model, P.m0);
+            ++n;
+            done = passed(L) | (n >= nmax);
+        }
+    if (WEIGHTED && lw != 0.0f) kahan_add(L.lw_hi, L.lw_lo, lw);
+    if (live && done) {
+        finish(P, L, n, passed(L));
+        live = false;
+    }
+    ++L.grp;
+}
+
+// Register budgets: two 512-thread blocks per SM (32 warps, at most 64
+// registers; direct sampling of 2^22 paths 46.1 ms with three blocks of 40
+// registers and guarded groups, 38.1 ms so); the learned-proposal steppers at most 384 threads per block and
+// two blocks, 80 registers: the network's fragments fit without spilling (a
+// 64-register build ran 512-thread blocks but executed ~7% more instructions
+// per step).
+template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET, bool RANK2>
+__device__ __forceinline__ void stepper(const EmParams &P)
 {
     extern __shared__ __align__(16) float4 s_tab[];
     __shared__ unsigned long long s_t0;
+    __shared__ TailSm s_tail;
 
+    // single-network MLP variants: the proposal's fragment blob follows the
+    // table in shared memory; then the run constants and model descriptors
     const int tab_entries = SMEM ? P.smem_table_points : 0;
     uint2 *s_tiles = reinterpret_cast<uint2 *>(s_tab + tab_entries);
     float *s_bias = reinterpret_cast<float *>(s_tiles + kMlpTiles * 32);
-    RunSm *s_run = smem_runs(s_tab, tab_entries, MLP);
+    RunSm *s_run = smem_runs(s_tab, tab_entries, MLP && !MNET);
     ModelDev *s_model = smem_models(s_run, P.n_runs);
     const RunDev &prun = P.runs[MLP ? P.mlp_run : 0];
-    stage_launch<SMEM, MLP>(P, s_tab, s_run, s_model, s_t0, s_tiles);
+    // units of the first chunks cover the launch: the tail starts at once
+    if (threadIdx.x == 0) s_tail.dry = (long long)gridDim.x * blockDim.x >= P.total_units;
+    stage_launch<SMEM, MLP && !MNET>(P, s_tab, s_run, s_model, s_t0, s_tiles);
 
     const float4 *tab = SMEM ? s_tab : P.tables;
     const unsigned FULL = 0xffffffffu;
+
     Lane L;
     SegRec sg;
     sg.open = false;
-    bool active = false, done = false;
-    first_units(P, L, active, s_run, s_model);
+    bool live = first_units(P, L, s_run, s_model);
+    bool tail = false;
+    int left = 0, round = 0;
 
     for (;;) {
-        if (MLP && __any_sync(FULL, active && L.mlp))
-            mlp2_segment_start<SMEM, REC>(L, active && L.mlp, sg, s_tiles, s_bias, prun, P.m0);
-
-        // speculative groups as in em_kernel, the precondition checked once per interval
-        bool spec = SMEM && __all_sync(FULL, active && !done &&
-                                                 L.n + 4 * P.groups_per_check < P.m0.max_steps);
-        for (int g = 0; g < P.groups_per_check; ++g) {
-            // four steps per group, two per Philox block: L.n is even at each block
-            // (a lane that finished keeps its count and ignores the normals).
-            // Speculative group as in em_kernel: when every lane is live and the
-            // interval stays below the cap, the steps run without the per-step
-            // branch and a lane that passed at step k of the group is set back to
-            // the guarded path's state (k + 1 steps, the weight and noise sums of
-            // those steps formed again from the same normals, field marked passed).
-            if (spec) {
-                const float sx0 = REC ? sg.sum_xi : 0.0f, sy0 = REC ? sg.sum_xi2 : 0.0f;
-                bool hit[4];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint4 r = philox4x32_10(make_uint4((uint32_t)L.n >> 1, L.traj, L.run_id, 0u), P.rk);
-                    float z[4];
-                    box_muller(r.x, r.y, z[0], z[1]);
-                    box_muller(r.z, r.w, z[2], z[3]);
-                    if (REC) { sg.sum_xi = __fadd_rn(sg.sum_xi, z[0]); sg.sum_xi2 = __fadd_rn(sg.sum_xi2, z[1]); }
-                    em2_step<WEIGHTED, SMEM, DTAB>(L, z[0], z[1], tab, s_model, P.m0);
-                    hit[2 * h] = passed(L);
-                    if (REC) { sg.sum_xi = __fadd_rn(sg.sum_xi, z[2]); sg.sum_xi2 = __fadd_rn(sg.sum_xi2, z[3]); }
-                    em2_step<WEIGHTED, SMEM, DTAB>(L, z[2], z[3], tab, s_model, P.m0);
-                    hit[2 * h + 1] = passed(L);
-                }
-                const bool any_hit = hit[0] | hit[1] | hit[2] | hit[3];
-                if (__any_sync(FULL, any_hit)) spec = false;
-                if (any_hit) {
-                    const int k = hit[0] ? 0 : hit[1] ? 1 : hit[2] ? 2 : 3;
-                    const int n0 = L.n - 4;
-                    float zz[8];
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const uint4 r = philox4x32_10(make_uint4(((uint32_t)n0 >> 1) + h, L.traj, L.run_id, 0u),
-                                                      P.rk);
-                        box_muller(r.x, r.y, zz[4 * h], zz[4 * h + 1]);
-                        box_muller(r.z, r.w, zz[4 * h + 2], zz[4 * h + 3]);
-                    }
-                    float lw = 0.0f, sx = sx0, sy = sy0;
-#pragma unroll
-                    for (int s = 0; s < 4; ++s) {
-                        if (s > k) break;
-                        lw -= fmaf(L.cb, zz[2 * s], fmaf(L.cb_b, zz[2 * s + 1], L.half_cb2));   // as em2_step
-                        sx = __fadd_rn(sx, zz[2 * s]);
-                        sy = __fadd_rn(sy, zz[2 * s + 1]);
-                    }
-                    L.n = n0 + k + 1;
-                    if (WEIGHTED) L.lw_grp = lw;
-                    if (REC) { sg.sum_xi = sx; sg.sum_xi2 = sy; }
-                    L.x = -1.0f;
-                    L.x_c = 0.0f;
-                    done = true;
+        if (__any_sync(FULL, live)) {
+            if (MLP && __any_sync(FULL, live && L.mlp)) {
+                if (RANK2) mlp2_segment_start<SMEM, REC>(L, live && L.mlp, sg, s_tiles, s_bias, prun, P.m0);
+                else if (MNET) mlp_segment_start_multi<SMEM, REC>(L, live && L.mlp, sg, tab, P.runs, P.m0);
+                else mlp_segment_start<SMEM, REC>(L, live && L.mlp, sg, tab, s_tiles, s_bias, prun, P.m0);
+            }
+            const int nmax = SMEM ? P.m0.max_steps : L.nmax;
+            if (__all_sync(FULL, !live || 4 * (L.grp + P.groups_per_check) <= nmax)) {
+                for (int g = 0; g < P.groups_per_check; ++g)
+                    run_group<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, tab, s_model);
+                if (live && 4 * L.grp >= nmax) {        // the cap falls on the interval's end
+                    finish(P, L, 4 * L.grp, false);
+                    live = false;
                 }
             } else {
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint4 r = philox4x32_10(make_uint4((uint32_t)L.n >> 1, L.traj, L.run_id, 0u), P.rk);
-                    float z[4];
-                    box_muller(r.x, r.y, z[0], z[1]);
-                    box_muller(r.z, r.w, z[2], z[3]);
-                    if (active && !done) {
-                        if (REC) { sg.sum_xi = __fadd_rn(sg.sum_xi, z[0]); sg.sum_xi2 = __fadd_rn(sg.sum_xi2, z[1]); }
-                        done = em2_step<WEIGHTED, SMEM, DTAB>(L, z[0], z[1], tab, s_model, P.m0);
-                    }
-                    if (active && !done) {
-                        if (REC) { sg.sum_xi = __fadd_rn(sg.sum_xi, z[2]); sg.sum_xi2 = __fadd_rn(sg.sum_xi2, z[3]); }
-                        done = em2_step<WEIGHTED, SMEM, DTAB>(L, z[2], z[3], tab, s_model, P.m0);
-                    }
-                }
+                for (int g = 0; g < P.groups_per_check; ++g)
+                    run_group_guarded<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, tab, s_model);
             }
-            if (WEIGHTED && L.lw_grp != 0.0f) {
-                kahan_add(L.lw_hi, L.lw_lo, L.lw_grp);
-                L.lw_grp = 0.0f;
-            }
+            if (REC) write_records<RANK2>(P, L, sg);
         }
-        // 2-D records: (inputs, sum xi_2), (0, sum xi_1, unit, steps)
-        if (REC) write_records(P, L, sg, active, make_float4(sg.in0, sg.in1, sg.in2, sg.sum_xi2), 0.0f, sg.sum_xi);
-        refill_point(P, L, active, done, s_run, s_model);
-        if (!__any_sync(FULL, active)) break;
-        if (P.budget_ns && past_deadline(P, s_t0)) break;
+        bool stop = false;
+        if (!tail) {
+            refill_point(P, L, live, s_run, s_model, &s_tail.dry);
+            // trajectories in flight keep the ABORTED status set before launch
+            stop = P.budget_ns && past_deadline(P, s_t0);
+            if (stop && (threadIdx.x & 31u) == 0) *(volatile int *)&s_tail.dry = 1;   // the others come to the meeting
+            __syncwarp();
+            if (!*(volatile int *)&s_tail.dry) continue;
+            tail = true;
+        } else {
+            if (--left > 0) continue;
+            stop = P.budget_ns && past_deadline(P, s_t0);
+        }
+        left = P.tail_intervals;
+        if (tail_meeting(P, L, live, stop, round++, s_tail, s_run, s_model) < 0) break;
     }
+}
+
+template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET = false>
+__global__ void __launch_bounds__(MLP ? kMlpMaxBlock : 512, 2) em_kernel(const EmParams P)
+{
+    stepper<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, false>(P);
+}
+
+template <bool WEIGHTED, bool SMEM, bool MLP, bool DTAB, bool REC = false>
+__global__ void __launch_bounds__(MLP ? kMlpMaxBlock : 512, 2) em2_kernel(const EmParams P)
+{
+    stepper<WEIGHTED, SMEM, MLP, REC, false, DTAB, false, true>(P);
 }
 
 template <bool DTAB>
