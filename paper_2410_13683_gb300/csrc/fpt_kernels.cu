@@ -444,7 +444,7 @@ __device__ __forceinline__ void mlp_segment_start(Lane &L, bool live, SegRec &sg
         tan_t = S > 0.0f ? __fdividef(T, S) : 0.0f;
     }
     float o1, o2;
-    mlp_forward_warp(tiles, bias, in0, in1, in2, o1, o2);
+    mlp_forward_warp(tiles, bias, in0, in1, in2, __ballot_sync(0xffffffffu, live), o1, o2);
     if (live) {
         float raw;
         const float al = mlp_alpha_of(o1, o2, tan_t, pr.alpha_max, raw);
@@ -491,7 +491,7 @@ __device__ __forceinline__ void mlp_segment_start_multi(Lane &L, bool live, SegR
         const uint2 *tiles = reinterpret_cast<const uint2 *>(pr.mlp);
         const float *bias = reinterpret_cast<const float *>(tiles + kMlpTiles * 32);
         float o1, o2;
-        mlp_forward_warp(tiles, bias, in0, in1, in2, o1, o2);
+        mlp_forward_warp(tiles, bias, in0, in1, in2, __ballot_sync(FULL, mine), o1, o2);
         if (mine) {
             float raw;
             const float al = mlp_alpha_of(o1, o2, tan_t, pr.alpha_max, raw);
@@ -824,7 +824,7 @@ __device__ __forceinline__ void mlp2_segment_start(Lane &L, bool live, SegRec &s
         in2 = ((float)(4 * L.grp) * dN - pr.shift[2]) * pr.scale[2];
     }
     float o1, o2;
-    mlp_forward_warp(tiles, bias, in0, in1, in2, o1, o2);
+    mlp_forward_warp(tiles, bias, in0, in1, in2, __ballot_sync(0xffffffffu, live), o1, o2);
     if (live) {
         const float b1 = fminf(fmaxf(o1, -pr.alpha_max), pr.alpha_max);
         const float b2 = fminf(fmaxf(o2, -pr.alpha_max), pr.alpha_max);

@@ -79,7 +79,7 @@ __global__ void mlp_eval_kernel(const uint2 *__restrict__ tiles, const float *__
         const bool ok = i < n;
         const float in0 = ok ? s[3 * i] : 0.0f, in1 = ok ? s[3 * i + 1] : 0.0f, in2 = ok ? s[3 * i + 2] : 0.0f;
         float o1, o2;
-        mlp_forward_warp(tiles, bias, in0, in1, in2, o1, o2);
+        mlp_forward_warp(tiles, bias, in0, in1, in2, 0xffffffffu, o1, o2);
         if (ok) {
             float raw;
             alpha[i] = mlp_alpha_of(o1, o2, tan_t[i], amax, raw);
@@ -289,8 +289,6 @@ __device__ __forceinline__ void ldsm_x4_trans(uint32_t &r0, uint32_t &r1, uint32
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(a));
 }
-
-__device__ __forceinline__ float sigmoid_f(float v) { return __fdividef(1.0f, 1.0f + __expf(-v)); }
 
 __device__ __forceinline__ float dsilu_f(float v)
 {
