@@ -1025,11 +1025,17 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
     const bool mlp = mlp_run >= 0;
     const EmVariant var{weighted, smem, mlp, mlp && ctx->record_mode, nidx && !mlp, rank2 == 1, bump == 1,
                         mlp && mnet};
-    const size_t smem_bytes = em_smem_bytes(var, smem ? ctx->region_entries[smem_model] : 0, n_runs,
-                                            (int)ctx->models.size());
+    const int entries = smem ? ctx->region_entries[smem_model] : 0, n_models = (int)ctx->models.size();
     // the learned-proposal steppers are compiled for at most kMlpMaxBlock threads
     const int block = mlp ? std::min(ctx->launch.block, kMlpMaxBlock) : ctx->launch.block;
-    int occ = em_occupancy(var, block, smem_bytes);
+    // the helper warps' rings take shared memory that the blocks per SM leave free
+    int pairs = em_max_pairs();
+    const int occ_plain = em_occupancy(var, block, em_smem_bytes(var, entries, n_runs, n_models, 0));
+    int occ = occ_plain;
+    while (pairs > 0 && (occ = em_occupancy(var, block, em_smem_bytes(var, entries, n_runs, n_models, pairs))) < occ_plain)
+        --pairs;
+    const size_t smem_bytes = em_smem_bytes(var, entries, n_runs, n_models, pairs);
+    if (pairs == 0) occ = em_occupancy(var, block, smem_bytes);   // the opt-in size of the launch
     if (occ < 1) return fail(ctx, FPT_E_CUDA, "stepper does not fit on an SM with this shape");
     const int bps = ctx->launch.blocks_per_sm ? std::min(ctx->launch.blocks_per_sm, occ) : occ;
     // no more blocks than chunks of 32 trajectories: a block's first warp takes a chunk each
@@ -1064,8 +1070,9 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
         }
     }
     p.groups_per_check = check_steps / 4;
-    p.tail_intervals = std::max(1, 128 / check_steps);
+    p.tail_intervals = std::max(1, 512 / check_steps);
     p.sm_count = ctx->sm_count;
+    p.pairs = pairs;
     p.mlp_run = mlp ? mlp_run : 0;
     p.records = ctx->d_records;
     p.rec_cursor = ctx->d_rec_cursor;

@@ -125,6 +125,7 @@ struct EmParams {
     int groups_per_check;      // refill every 4 * groups_per_check steps
     int tail_intervals;        // intervals between two meetings of a block's warps in the launch's tail
     int sm_count;
+    int pairs;                 // rings for helper warps in the block's shared memory
     unsigned long long budget_ns;    // > 0: abort after this long (device clock)
     unsigned long long *t0;          // first %globaltimer reading of the launch (0 before)
     // learned proposal (MLP variants): launch-wide proposal, from the first MLP run
@@ -167,7 +168,8 @@ struct EmVariant {
 
 // Host wrappers implemented in fpt_kernels.cu.
 int em_occupancy(EmVariant v, int block, size_t smem_bytes);
-size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models);
+size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models, int pairs);
+int em_max_pairs();
 // FPT_CHECKS builds: read and clear the device error word of the bounds checks
 // (kCheck* bits; synchronous). Other builds return 0.
 cudaError_t checks_take(int *word);

@@ -507,9 +507,27 @@ __device__ __forceinline__ void mlp_segment_start_multi(Lane &L, bool live, SegR
     }
 }
 
+// Shared memory of the launch's tail (see tail_meeting).
+constexpr int kPoolLanes = 128;          // lanes one compaction can move (4 KB of shared memory)
+constexpr int kMaxWarps = 16;
+constexpr int kMaxPairs = 4;             // warps of a block that can have a helper
+constexpr int kSlotVecs = 4 * 32;        // float4 of a ring slot: four Philox blocks of 32 lanes
+
+struct PairSm {
+    float4 ring[2 * kSlotVecs];
+    uint4 lane[32];                      // generator state of the consumer's lanes, next group
+};
+
+struct TailSm {
+    float4 pool[2 * kPoolLanes];
+    int count[2][kMaxWarps];             // live lanes per warp, double-buffered by round
+    int dry;
+};
+
 // Dynamic shared memory of a stepper launch: the table (SMEM variants), the
 // staged proposal blob (single-network learned variants), then the launch's
-// run constants and model descriptors, each as many as the launch has.
+// run constants and model descriptors, each as many as the launch has, and the
+// rings of the tail's helper warps.
 __device__ __forceinline__ RunSm *smem_runs(float4 *s_dyn, int table_entries, bool staged_blob)
 {
     unsigned char *p = reinterpret_cast<unsigned char *>(s_dyn + table_entries);
@@ -522,10 +540,11 @@ __device__ __forceinline__ ModelDev *smem_models(RunSm *s_run, int n_runs)
     return reinterpret_cast<ModelDev *>(reinterpret_cast<unsigned char *>(s_run) + b);
 }
 
-size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models)
+
+__device__ __forceinline__ PairSm *smem_pairs(ModelDev *s_model, int n_models)
 {
-    return sizeof(float4) * (size_t)table_entries + ((v.mlp && !v.mnet) ? (size_t)kMlpBlobBytes : 0) +
-           ((sizeof(RunSm) * (size_t)n_runs + 15) / 16) * 16 + sizeof(ModelDev) * (size_t)n_models;
+    const size_t b = ((sizeof(ModelDev) * (size_t)n_models + 15) / 16) * 16;
+    return reinterpret_cast<PairSm *>(reinterpret_cast<unsigned char *>(s_model) + b);
 }
 
 // Launch prologue shared by the steppers: clock origin, per-run and per-model
@@ -589,7 +608,7 @@ __device__ __forceinline__ void finish(const EmParams &P, const Lane &L, int n, 
 // sub-partitions.
 __device__ __forceinline__ int block_rotation(const EmParams &P)
 {
-    return (int)((blockIdx.x / (unsigned)P.sm_count) % (blockDim.x >> 5));
+    return (int)(2 * (blockIdx.x / (unsigned)P.sm_count) % (blockDim.x >> 5));
 }
 
 __device__ __forceinline__ bool first_units(const EmParams &P, Lane &L, const RunSm *s_run,
@@ -646,13 +665,15 @@ __device__ __forceinline__ bool refill_point(const EmParams &P, Lane &L, bool &l
 // with the straight-line groups below: 2^18 learned paths (median 8,902 steps,
 // longest 262,144) 78 -> 34 ms, where the longest path's step took 324 ns
 // among 24 sparse warps per SM; 64 models x 8,192 paths 76 -> 32 ms.
-constexpr int kPoolLanes = 128;          // lanes one compaction can move (4 KB of shared memory)
-constexpr int kMaxWarps = 16;
-
-struct TailSm {
-    float4 pool[2 * kPoolLanes];
-    int count[2][kMaxWarps];             // live lanes per warp, double-buffered by round
-    int dry;
+//
+// When few warps are left, each gets an idle warp of its block as a helper that
+// draws its normals: a lone warp takes ~150 cycles a step, of which its own
+// chain (field -> table -> field) is about 85 and a third of the instructions
+// are the generator's. The helper keeps one slot ahead in a ring of two slots
+// in shared memory; the two warps meet at a named barrier per slot.
+struct TailRole {
+    int pair;                            // index of the warp's ring, -1: none
+    bool helper;
 };
 
 __device__ __forceinline__ int warp_at(int pos, int rot, int nw)
@@ -661,63 +682,86 @@ __device__ __forceinline__ int warp_at(int pos, int rot, int nw)
     return w >= nw ? w - nw : w;
 }
 
-// One meeting of the block's warps. Returns -1 when the block has no live lane
-// left (or must stop), else 1 when this warp's lanes changed, 0 when not.
-__device__ __forceinline__ int tail_meeting(const EmParams &P, Lane &L, bool &live, bool stop, int round,
-                                            TailSm &T, const RunSm *s_run, const ModelDev *s_model)
+__device__ __forceinline__ int scan_incl(int v)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < kMaxWarps; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += u;
+    }
+    return v;
+}
+
+// One meeting of the block's warps. Returns false when the block has no live
+// lane left or must stop. Lane j of every warp holds the count of the warp at
+// position j, so all warps come to the same decision.
+__device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &live, bool stop, int round,
+                                             TailSm &T, PairSm *pairs, const RunSm *s_run,
+                                             const ModelDev *s_model, TailRole &role)
 {
     const unsigned FULL = 0xffffffffu;
-    const unsigned lane = threadIdx.x & 31u;
-    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5, rot = block_rotation(P);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int rot = block_rotation(P), pos = warp_at(warp, nw - rot, nw);
     const unsigned mask = __ballot_sync(FULL, live);
     int *cnt = T.count[round & 1];
     if (lane == 0) cnt[warp] = __popc(mask);
-    if (__syncthreads_or(stop)) return -1;
-    int total = 0, used = 0;
-    for (int j = 0; j < nw; ++j) {
-        total += cnt[j];
-        used += cnt[j] > 0;
-    }
-    if (!total) return -1;
-    // keep the first `keep` positions; the later ones' lanes must fit the pool
-    int keep = nw, moved = 0;
+    if (__syncthreads_or(stop)) return false;
+    const int c = lane < nw ? cnt[warp_at(lane, rot, nw)] : 0;
+    const int total = __reduce_add_sync(FULL, c);
+    if (!total) return false;
+    unsigned busy = __ballot_sync(FULL, c > 0);
     const int need = (total + 31) >> 5;
-    if (need < used) {
-        while (keep > need && moved + cnt[warp_at(keep - 1, rot, nw)] <= kPoolLanes)
-            moved += cnt[warp_at(--keep, rot, nw)];
-    }
-    if (!moved) return 0;
-    // donors in order of position fill the pool, free lanes in the same order empty it
-    int before = 0, pos = 0;
-    for (int j = 0; j < nw; ++j) {
-        const int w = warp_at(j, rot, nw);
-        if (w == warp) { pos = j; break; }
-        if (j < keep) before += 32 - cnt[w];
-    }
-    const bool donor = pos >= keep;
-    if (donor) {
-        before = 0;
-        for (int j = keep; j < pos; ++j) before += cnt[warp_at(j, rot, nw)];
-        if (live) {
-            const int e = before + __popc(mask & ((1u << lane) - 1u));
-            T.pool[2 * e] = make_float4(L.x, L.x_c, L.p, L.p_c);
-            T.pool[2 * e + 1] = make_float4(L.lw_hi, L.lw_lo, __int_as_float(L.grp), __uint_as_float(L.unit));
-            live = false;
+    if (need < __popc(busy)) {
+        // keep the first positions; the lanes of the later ones must fit the pool
+        const int excl = scan_incl(c) - c;
+        const unsigned fits = __ballot_sync(FULL, lane >= need && lane < nw && total - excl <= kPoolLanes);
+        const int keep = fits ? __ffs(fits) - 1 : nw;
+        const int moved = fits ? total - __shfl_sync(FULL, excl, keep & 31) : 0;
+        if (moved) {
+            // donors in order of position fill the pool, free lanes in the same order empty it
+            const int room = lane < keep ? 32 - c : 0;
+            const int room_excl = scan_incl(room) - room;
+            const bool donor = pos >= keep;
+            const int from = __shfl_sync(FULL, excl, pos) - (total - moved), to = __shfl_sync(FULL, room_excl, pos);
+            busy = __ballot_sync(FULL, lane < keep && (c > 0 || (room > 0 && room_excl < moved)));
+            const unsigned below = (1u << lane) - 1u;
+            if (donor && live) {
+                const int e = from + __popc(mask & below);
+                T.pool[2 * e] = make_float4(L.x, L.x_c, L.p, L.p_c);
+                T.pool[2 * e + 1] = make_float4(L.lw_hi, L.lw_lo, __int_as_float(L.grp), __uint_as_float(L.unit));
+                live = false;
+            }
+            __syncthreads();
+            const int e = to + __popc(~mask & below);
+            const bool take = !donor && !live && e < moved;
+            if (take) {
+                const float4 u = T.pool[2 * e], v = T.pool[2 * e + 1];
+                lane_load(L, (long long)__float_as_uint(v.w), s_run, s_model, P.n_runs, P.rk);
+                L.x = u.x; L.x_c = u.y; L.p = u.z; L.p_c = u.w;
+                L.lw_hi = v.x; L.lw_lo = v.y;
+                L.grp = __float_as_int(v.z);
+                live = true;
+            }
         }
     }
-    __syncthreads();
-    if (donor) return 0;
-    const int e = before + __popc(~mask & ((1u << lane) - 1u));
-    const bool take = !live && e < moved;
-    if (take) {
-        const float4 a = T.pool[2 * e], b = T.pool[2 * e + 1];
-        lane_load(L, (long long)__float_as_uint(b.w), s_run, s_model, P.n_runs, P.rk);
-        L.x = a.x; L.x_c = a.y; L.p = a.z; L.p_c = a.w;
-        L.lw_hi = b.x; L.lw_lo = b.y;
-        L.grp = __float_as_int(b.z);
-        live = true;
+    // helpers for the busy warps, if there are few enough
+    const int n_busy = __popc(busy);
+    role.pair = -1;
+    if (n_busy <= P.pairs && 2 * n_busy <= nw) {
+        const unsigned below = (1u << pos) - 1u;
+        role.helper = !((busy >> pos) & 1u);
+        const int rank = __popc((role.helper ? ~busy : busy) & below);
+        if (rank < n_busy) role.pair = rank;
+        if (!role.helper) pairs[rank].lane[lane] = make_uint4(L.rng.a, L.rng.b, L.rng.c, (uint32_t)L.grp);
+        __syncthreads();
     }
-    return __any_sync(FULL, take) ? 1 : 0;
+    return true;
+}
+
+__device__ __forceinline__ void pair_barrier(int pair)
+{
+    asm volatile("bar.sync %0, 64;" ::"r"(pair + 1) : "memory");
 }
 
 // Deadline: true when the launch should stop (lane 0 reads the device clock).
@@ -857,13 +901,61 @@ __device__ __forceinline__ void any_step(Lane &L, int n, int s, const float *z, 
 // Normals of group grp: Philox block grp (1-D noise: one normal per step), blocks
 // 2 grp and 2 grp + 1 (full-rank noise: two per step).
 template <bool RANK2>
-__device__ __forceinline__ void group_normals(const EmParams &P, const Lane &L, int grp, float *z)
+__device__ __forceinline__ void group_normals(const EmParams &P, const PhiloxLane &rng, int grp, float *z)
 {
 #pragma unroll
     for (int h = 0; h < (RANK2 ? 2 : 1); ++h) {
-        const uint4 r = philox4x32_10((RANK2 ? 2u : 1u) * (uint32_t)grp + h, L.rng, P.rk);
+        const uint4 r = philox4x32_10((RANK2 ? 2u : 1u) * (uint32_t)grp + h, rng, P.rk);
         box_muller(r.x, r.y, z[4 * h], z[4 * h + 1]);
         box_muller(r.z, r.w, z[4 * h + 2], z[4 * h + 3]);
+    }
+}
+
+// Ring of normals between a helper warp and its consumer: slots of four Philox
+// blocks. The helper passes the slot's barrier when it has filled the slot, the
+// consumer when it starts on it (and has read the one before).
+template <bool RANK2>
+struct Ring {
+    static constexpr int kGroups = RANK2 ? 2 : 4;
+    PairSm *pair;
+    int index, g;                        // pair index, groups consumed
+
+    __device__ __forceinline__ void skip()
+    {
+        if (g % kGroups == 0) pair_barrier(index);
+        ++g;
+    }
+    __device__ __forceinline__ void take(float *z)
+    {
+        const float4 *q = pair->ring + (g & (2 * kGroups - 1)) * (RANK2 ? 64 : 32) + (threadIdx.x & 31);
+        skip();
+#pragma unroll
+        for (int h = 0; h < (RANK2 ? 2 : 1); ++h) {
+            const float4 v = q[32 * h];
+            z[4 * h] = v.x; z[4 * h + 1] = v.y; z[4 * h + 2] = v.z; z[4 * h + 3] = v.w;
+        }
+    }
+};
+
+// The helper's part: normals of `groups` groups of the consumer's lanes.
+template <bool RANK2>
+__device__ __forceinline__ void help(const EmParams &P, PairSm &pair, int index, int groups)
+{
+    constexpr int kGroups = Ring<RANK2>::kGroups;
+    const int lane = threadIdx.x & 31;
+    const uint4 q = pair.lane[lane];
+    const PhiloxLane rng = {q.x, q.y, q.z};
+    for (int g = 0; g < groups; g += kGroups) {
+        float4 *slot = pair.ring + (g & (2 * kGroups - 1)) * (RANK2 ? 64 : 32) + lane;
+#pragma unroll
+        for (int k = 0; k < kGroups; ++k) {
+            float z[RANK2 ? 8 : 4];
+            group_normals<RANK2>(P, rng, (int)q.w + g + k, z);
+#pragma unroll
+            for (int h = 0; h < (RANK2 ? 2 : 1); ++h)
+                slot[32 * ((RANK2 ? 2 : 1) * k + h)] = make_float4(z[4 * h], z[4 * h + 1], z[4 * h + 2], z[4 * h + 3]);
+        }
+        pair_barrier(index);
     }
 }
 
@@ -888,11 +980,9 @@ __device__ __forceinline__ void add_xi(SegRec &sg, const float *z, int k)
 // every table index is clamped, so it stays in bounds. A warp with idle lanes
 // thus runs the same straight code as a full one.
 template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
-__device__ __forceinline__ void run_group(const EmParams &P, Lane &L, bool &live, SegRec &sg,
+__device__ __forceinline__ void run_group(const EmParams &P, Lane &L, bool &live, SegRec &sg, const float *z,
                                           const float4 *__restrict__ tab, const ModelDev *s_model)
 {
-    float z[RANK2 ? 8 : 4];
-    group_normals<RANK2>(P, L, L.grp, z);
     const int n0 = 4 * L.grp;
     float lw = 0.0f;
     bool h[4];
@@ -926,10 +1016,9 @@ __device__ __forceinline__ void run_group(const EmParams &P, Lane &L, bool &live
 // reaches the step cap inside a group.
 template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
 __device__ __forceinline__ void run_group_guarded(const EmParams &P, Lane &L, bool &live, SegRec &sg,
-                                                  const float4 *__restrict__ tab, const ModelDev *s_model)
+                                                  const float *z, const float4 *__restrict__ tab,
+                                                  const ModelDev *s_model)
 {
-    float z[RANK2 ? 8 : 4];
-    group_normals<RANK2>(P, L, L.grp, z);
     const int nmax = SMEM ? P.m0.max_steps : L.nmax;
     int n = 4 * L.grp;
     float lw = 0.0f;
@@ -953,6 +1042,47 @@ __device__ __forceinline__ void run_group_guarded(const EmParams &P, Lane &L, bo
     ++L.grp;
 }
 
+// One interval of the warp: the proposal's evaluation, the groups, the records.
+template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET, bool RANK2, bool RING>
+__device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &live, SegRec &sg, Ring<RANK2> &ring,
+                                             const float4 *__restrict__ tab, const RunSm *s_run,
+                                             const ModelDev *s_model, const uint2 *s_tiles, const float *s_bias,
+                                             const RunDev &prun)
+{
+    const unsigned FULL = 0xffffffffu;
+    if (!__any_sync(FULL, live)) {
+        if (RING)
+            for (int g = 0; g < P.groups_per_check; ++g) ring.skip();
+        return;
+    }
+    if (MLP && __any_sync(FULL, live && L.mlp)) {
+        if (RANK2) mlp2_segment_start<SMEM, REC>(L, live && L.mlp, sg, s_tiles, s_bias, prun, P.m0);
+        else if (MNET) mlp_segment_start_multi<SMEM, REC>(L, live && L.mlp, sg, tab, P.runs, P.m0);
+        else mlp_segment_start<SMEM, REC>(L, live && L.mlp, sg, tab, s_tiles, s_bias, prun, P.m0);
+    }
+    const int nmax = SMEM ? P.m0.max_steps : L.nmax;
+    const bool capped_inside = __any_sync(FULL, live && 4 * (L.grp + P.groups_per_check) > nmax);
+    float z[RANK2 ? 8 : 4];
+    if (!capped_inside) {
+        for (int g = 0; g < P.groups_per_check; ++g) {
+            if (RING) ring.take(z);
+            else group_normals<RANK2>(P, L.rng, L.grp, z);
+            run_group<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, z, tab, s_model);
+        }
+        if (live && 4 * L.grp >= nmax) {        // the cap falls on the interval's end
+            finish(P, L, 4 * L.grp, false);
+            live = false;
+        }
+    } else {
+        for (int g = 0; g < P.groups_per_check; ++g) {
+            if (RING) ring.skip();
+            group_normals<RANK2>(P, L.rng, L.grp, z);
+            run_group_guarded<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, z, tab, s_model);
+        }
+    }
+    if (REC) write_records<RANK2>(P, L, sg);
+}
+
 // Register budgets: two 512-thread blocks per SM (32 warps, at most 64
 // registers; direct sampling of 2^22 paths 46.1 ms with three blocks of 40
 // registers and guarded groups, 38.1 ms so); the learned-proposal steppers at most 384 threads per block and
@@ -973,57 +1103,46 @@ __device__ __forceinline__ void stepper(const EmParams &P)
     float *s_bias = reinterpret_cast<float *>(s_tiles + kMlpTiles * 32);
     RunSm *s_run = smem_runs(s_tab, tab_entries, MLP && !MNET);
     ModelDev *s_model = smem_models(s_run, P.n_runs);
+    PairSm *s_pairs = smem_pairs(s_model, P.n_models);
     const RunDev &prun = P.runs[MLP ? P.mlp_run : 0];
     // units of the first chunks cover the launch: the tail starts at once
     if (threadIdx.x == 0) s_tail.dry = (long long)gridDim.x * blockDim.x >= P.total_units;
     stage_launch<SMEM, MLP && !MNET>(P, s_tab, s_run, s_model, s_t0, s_tiles);
 
     const float4 *tab = SMEM ? s_tab : P.tables;
-    const unsigned FULL = 0xffffffffu;
 
     Lane L;
     SegRec sg;
     sg.open = false;
     bool live = first_units(P, L, s_run, s_model);
-    bool tail = false;
-    int left = 0, round = 0;
-
-    for (;;) {
-        if (__any_sync(FULL, live)) {
-            if (MLP && __any_sync(FULL, live && L.mlp)) {
-                if (RANK2) mlp2_segment_start<SMEM, REC>(L, live && L.mlp, sg, s_tiles, s_bias, prun, P.m0);
-                else if (MNET) mlp_segment_start_multi<SMEM, REC>(L, live && L.mlp, sg, tab, P.runs, P.m0);
-                else mlp_segment_start<SMEM, REC>(L, live && L.mlp, sg, tab, s_tiles, s_bias, prun, P.m0);
-            }
-            const int nmax = SMEM ? P.m0.max_steps : L.nmax;
-            if (__all_sync(FULL, !live || 4 * (L.grp + P.groups_per_check) <= nmax)) {
-                for (int g = 0; g < P.groups_per_check; ++g)
-                    run_group<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, tab, s_model);
-                if (live && 4 * L.grp >= nmax) {        // the cap falls on the interval's end
-                    finish(P, L, 4 * L.grp, false);
-                    live = false;
-                }
-            } else {
-                for (int g = 0; g < P.groups_per_check; ++g)
-                    run_group_guarded<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, tab, s_model);
-            }
-            if (REC) write_records<RANK2>(P, L, sg);
-        }
-        bool stop = false;
-        if (!tail) {
-            refill_point(P, L, live, s_run, s_model, &s_tail.dry);
-            // trajectories in flight keep the ABORTED status set before launch
-            stop = P.budget_ns && past_deadline(P, s_t0);
-            if (stop && (threadIdx.x & 31u) == 0) *(volatile int *)&s_tail.dry = 1;   // the others come to the meeting
-            __syncwarp();
-            if (!*(volatile int *)&s_tail.dry) continue;
-            tail = true;
+    Ring<RANK2> ring{};
+    // until the work is dealt out: an interval, then new trajectories for the idle lanes
+    bool stop = false;
+    while (!*(volatile int *)&s_tail.dry) {
+        run_interval<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, RANK2, false>(P, L, live, sg, ring, tab, s_run,
+                                                                              s_model, s_tiles, s_bias, prun);
+        refill_point(P, L, live, s_run, s_model, &s_tail.dry);
+        // trajectories in flight keep the ABORTED status set before launch
+        stop = P.budget_ns && past_deadline(P, s_t0);
+        if (stop && (threadIdx.x & 31u) == 0) *(volatile int *)&s_tail.dry = 1;   // the others come to the meeting
+        __syncwarp();
+    }
+    // the tail
+    TailRole role;
+    for (int round = 0; tail_meeting(P, L, live, stop, round, s_tail, s_pairs, s_run, s_model, role); ++round) {
+        if (role.pair < 0) {
+            for (int k = 0; k < P.tail_intervals; ++k)
+                run_interval<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, RANK2, false>(
+                    P, L, live, sg, ring, tab, s_run, s_model, s_tiles, s_bias, prun);
+        } else if (role.helper) {
+            help<RANK2>(P, s_pairs[role.pair], role.pair, P.tail_intervals * P.groups_per_check);
         } else {
-            if (--left > 0) continue;
-            stop = P.budget_ns && past_deadline(P, s_t0);
+            ring = Ring<RANK2>{s_pairs + role.pair, role.pair, 0};
+            for (int k = 0; k < P.tail_intervals; ++k)
+                run_interval<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, RANK2, true>(
+                    P, L, live, sg, ring, tab, s_run, s_model, s_tiles, s_bias, prun);
         }
-        left = P.tail_intervals;
-        if (tail_meeting(P, L, live, stop, round++, s_tail, s_run, s_model) < 0) break;
+        stop = P.budget_ns && past_deadline(P, s_t0);
     }
 }
 
@@ -1079,6 +1198,15 @@ static const void *em_fn(EmVariant v)
     }
     return em_fn_t<false>(v);
 }
+
+size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models, int pairs)
+{
+    return sizeof(float4) * (size_t)table_entries + ((v.mlp && !v.mnet) ? (size_t)kMlpBlobBytes : 0) +
+           ((sizeof(RunSm) * (size_t)n_runs + 15) / 16) * 16 + ((sizeof(ModelDev) * (size_t)n_models + 15) / 16) * 16 +
+           sizeof(PairSm) * (size_t)pairs;
+}
+
+int em_max_pairs() { return kMaxPairs; }
 
 // Opt in to the dynamic shared memory the table (and proposal) need, outside
 // any stream capture, then report resident blocks per SM for this shape.
