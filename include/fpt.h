@@ -509,7 +509,7 @@ fpt_status fpt_run_records(fpt_ctx *ctx, const fpt_run_desc *run, int64_t cap, f
  * an interface variant, not a step of the method.
  *
  * No context, no allocation: the scratch (per-bin maxima, jackknife moments,
- * scalars; about 1.3 MB) is a fixed array inside the library that every GPU
+ * scalars; about 1.4 MB) is a fixed array inside the library that every GPU
  * loading the library holds until the process exits. The call runs in the
  * CUDA context current on the calling thread (with none current, the current
  * device's primary context). The array's device address is valid only in

@@ -85,9 +85,7 @@ struct fpt_ctx {
     long long unit_cap = 0;
 
     // histogram scratch
-    unsigned long long *d_hmax = nullptr;
-    double *d_hmom = nullptr;
-    double *d_hscal = nullptr;
+    unsigned char *d_hist = nullptr;
     double *d_hout = nullptr;
     double *h_hout = nullptr;
     // caller-data histogram scratch
@@ -237,9 +235,7 @@ static void free_all(fpt_ctx *ctx)
     dev_free(ctx, ctx->d_logw);
     dev_free(ctx, ctx->d_status);
     dev_free(ctx, ctx->d_N);
-    dev_free(ctx, ctx->d_hmax);
-    dev_free(ctx, ctx->d_hmom);
-    dev_free(ctx, ctx->d_hscal);
+    dev_free(ctx, ctx->d_hist);
     dev_free(ctx, ctx->d_hout);
     cudaFreeHost(ctx->h_hout);
     dev_free(ctx, ctx->d_records);
@@ -616,9 +612,7 @@ fpt_status fpt_init_model(fpt_ctx **pctx, const fpt_model *models, int32_t n_mod
     if ((e = dev_malloc(ctx, &ctx->d_cursor, 64))) return bail(e, "cudaMalloc cursor");
     if ((e = dev_malloc(ctx, &ctx->d_flags, 64))) return bail(e, "cudaMalloc flags");
     if ((e = cudaMallocHost(&ctx->h_flags, 64))) return bail(e, "cudaMallocHost flags");
-    if ((e = dev_malloc(ctx, &ctx->d_hmax, sizeof(unsigned long long) * (kMaxBins + 2)))) return bail(e, "cudaMalloc hist");
-    if ((e = dev_malloc(ctx, &ctx->d_hmom, sizeof(double) * (size_t)kJackknife * kMaxBins * 5))) return bail(e, "cudaMalloc hist");
-    if ((e = dev_malloc(ctx, &ctx->d_hscal, sizeof(double) * kJackknife * 16))) return bail(e, "cudaMalloc hist");
+    if ((e = dev_malloc(ctx, &ctx->d_hist, hist_scratch_bytes(kMaxBins)))) return bail(e, "cudaMalloc hist");
     if ((e = dev_malloc(ctx, &ctx->d_hout, sizeof(double) * hout_doubles()))) return bail(e, "cudaMalloc hist");
     if ((e = cudaMallocHost(&ctx->h_hout, sizeof(double) * hout_doubles()))) return bail(e, "cudaMallocHost hist");
     std::memset(ctx->h_flags, 0, 64);
@@ -1222,10 +1216,7 @@ static fpt_status hist_run(fpt_ctx *ctx, const int32_t *nsteps, const double *lo
     p.db = (N_hi - N_lo) / n_bins;
     p.N_tail = N_tail;
     p.n_bins = n_bins;
-    p.chunk = 4096;
-    p.maxkey = ctx->d_hmax;
-    p.mom = ctx->d_hmom;
-    p.scal = ctx->d_hscal;
+    p.scratch = ctx->d_hist;
     cudaError_t e = hist_launch(p, ctx->d_hout, s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "histogram launch");
     const size_t nd = (size_t)10 * n_bins + 16;
@@ -1786,7 +1777,6 @@ fpt_status fpt_histogram_noalloc(const int32_t *nsteps, const double *logw, cons
     p.db = (N_hi - N_lo) / n_bins;
     p.N_tail = N_tail;
     p.n_bins = n_bins;
-    p.chunk = 4096;
     cudaError_t e = hist_noalloc_launch(p, out, (cudaStream_t)cuda_stream);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "fpt_histogram_noalloc");
     return FPT_OK;

@@ -145,16 +145,8 @@ struct HistParams {
     double dN;
     double N_lo, db, N_tail;   // N_tail NaN: no tail set
     int n_bins;
-    int chunk;                 // units per CTA
-    unsigned long long *maxkey;   // [n_bins + 2]: per-bin, global, tail max of ln w
-    double *mom;               // [kJackknife][n_bins][5]: count, S1, S2, Slw, Slw2
-    double *scal;              // [kJackknife][16] scalars
-};
-
-// Scalar slots of HistParams::scal (per jackknife block).
-enum {
-    kScN = 0, kScPassed, kScUnder, kScOver, kScCapped, kScSumN, kScSumWN, kScSumW,
-    kScTailW, kScTailW2, kScTailN, kScCount
+    long long chunk;           // units per CTA of the summing kernel
+    unsigned char *scratch;    // hist_scratch_bytes(n_bins) bytes, 64-byte aligned
 };
 
 // Stepper variants: weighted (any bias), table in shared memory, learned
@@ -195,6 +187,7 @@ size_t mlp_bwd_smem();
 cudaError_t hist_launch(const HistParams &p, double *out, cudaStream_t s);
 cudaError_t hist_noalloc_launch(HistParams p, double *out, cudaStream_t s);
 size_t hist_noalloc_scratch_bytes();
+size_t hist_scratch_bytes(int n_bins);
 cudaError_t n_of_steps_launch(const int32_t *nsteps, long long n, double dN, double *N,
                               cudaStream_t s);
 
