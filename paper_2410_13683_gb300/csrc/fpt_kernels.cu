@@ -694,8 +694,15 @@ __device__ __forceinline__ int scan_incl(int v)
 }
 
 // One meeting of the block's warps. Returns false when the block has no live
-// lane left or must stop. Lane j of every warp holds the count of the warp at
+// lane left or must stop. kMinWarps: warps that compaction leaves busy if it can,
+// the lanes spread evenly over them. A warp with one network per run evaluates
+// the networks of its lanes in turn, so its lanes are spread over eight warps
+// (training round of 64 networks, 1,024 paths each: 26.7 ms with one, 24.4 with
+// two, 22.7 with eight); a step costs a warp the same for one lane and for 32,
+// so the others are better packed (2^18 learned paths: 30.3 ms with one, 33.2
+// with four, 47.7 with eight). Lane j of every warp holds the count of the warp at
 // position j, so all warps come to the same decision.
+template <int kMinWarps>
 __device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &live, bool stop, int round,
                                              TailSm &T, PairSm *pairs, const RunSm *s_run,
                                              const ModelDev *s_model, TailRole &role)
@@ -711,7 +718,7 @@ __device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &l
     const int total = __reduce_add_sync(FULL, c);
     if (!total) return false;
     unsigned busy = __ballot_sync(FULL, c > 0);
-    const int need = (total + 31) >> 5;
+    const int need = max((total + 31) >> 5, min(kMinWarps, nw));
     if (need < __popc(busy)) {
         // keep the first positions; the lanes of the later ones must fit the pool
         const int excl = scan_incl(c) - c;
@@ -720,7 +727,7 @@ __device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &l
         const int moved = fits ? total - __shfl_sync(FULL, excl, keep & 31) : 0;
         if (moved) {
             // donors in order of position fill the pool, free lanes in the same order empty it
-            const int room = lane < keep ? 32 - c : 0;
+            const int room = lane < keep ? max(0, (total + keep - 1) / keep - c) : 0;
             const int room_excl = scan_incl(room) - room;
             const bool donor = pos >= keep;
             const int from = __shfl_sync(FULL, excl, pos) - (total - moved), to = __shfl_sync(FULL, room_excl, pos);
@@ -733,8 +740,8 @@ __device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &l
                 live = false;
             }
             __syncthreads();
-            const int e = to + __popc(~mask & below);
-            const bool take = !donor && !live && e < moved;
+            const int free = __popc(~mask & below), mine = __shfl_sync(FULL, room, pos), e = to + free;
+            const bool take = !donor && !live && free < mine && e < moved;
             if (take) {
                 const float4 u = T.pool[2 * e], v = T.pool[2 * e + 1];
                 lane_load(L, (long long)__float_as_uint(v.w), s_run, s_model, P.n_runs, P.rk);
@@ -1129,7 +1136,8 @@ __device__ __forceinline__ void stepper(const EmParams &P)
     }
     // the tail
     TailRole role;
-    for (int round = 0; tail_meeting(P, L, live, stop, round, s_tail, s_pairs, s_run, s_model, role); ++round) {
+    for (int round = 0;
+         tail_meeting<MNET ? 8 : 1>(P, L, live, stop, round, s_tail, s_pairs, s_run, s_model, role); ++round) {
         if (role.pair < 0) {
             for (int k = 0; k < P.tail_intervals; ++k)
                 run_interval<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, RANK2, false>(

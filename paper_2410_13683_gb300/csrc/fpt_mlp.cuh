@@ -76,68 +76,97 @@ __device__ __forceinline__ float silu_f(float v)
     return v * sigmoid_f(v);
 }
 
+// One M tile: row g of the tile is the state of lane src0, row g + 8 that of
+// lane src1. EIGHT: only the first eight rows are used (and their activations
+// formed). Lane 4 g ends with row g's outputs in d3[0..1], row g + 8's in d3[2..3].
+template <bool EIGHT>
+__device__ __forceinline__ void mlp_tile(const uint2 *tiles, const float *bias, float in0, float in1, float in2,
+                                         int src0, int src1, float d3[4])
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, t = lane & 3;
+    const float *b1 = bias, *b2 = bias + kMlpH, *b3 = bias + 2 * kMlpH;
+    const float x0 = __shfl_sync(FULL, in0, src0), y0 = __shfl_sync(FULL, in1, src0), z0 = __shfl_sync(FULL, in2, src0);
+    // layer-1 A fragment: row r, columns (2t, 2t+1) of (s0, s1, s2, 0, ..., 0)
+    const uint32_t a0 = pack_bf16x2(t == 0 ? x0 : (t == 1 ? z0 : 0.0f), t == 0 ? y0 : 0.0f);
+    uint32_t a1 = 0u;
+    if (!EIGHT) {
+        const float x1 = __shfl_sync(FULL, in0, src1), y1 = __shfl_sync(FULL, in1, src1), z1 = __shfl_sync(FULL, in2, src1);
+        a1 = pack_bf16x2(t == 0 ? x1 : (t == 1 ? z1 : 0.0f), t == 0 ? y1 : 0.0f);
+    }
+    auto act = [](const float *d, uint32_t &lo, uint32_t &hi) {
+        lo = pack_bf16x2(silu_f(d[0]), silu_f(d[1]));
+        hi = EIGHT ? 0u : pack_bf16x2(silu_f(d[2]), silu_f(d[3]));
+    };
+    // layer 1, two N tiles at a time -> the four K tiles of layer 2's A operand
+    uint32_t A[4][4];
+#pragma unroll
+    for (int kt = 0; kt < 4; ++kt) {
+        const float2 c0 = *reinterpret_cast<const float2 *>(b1 + 16 * kt + 2 * t);
+        const float2 c1 = *reinterpret_cast<const float2 *>(b1 + 16 * kt + 8 + 2 * t);
+        float d0[4] = {c0.x, c0.y, c0.x, c0.y}, d1[4] = {c1.x, c1.y, c1.x, c1.y};
+        mma_bf16_16816(d0, a0, a1, 0u, 0u, tiles[(2 * kt) * 32 + lane]);
+        mma_bf16_16816(d1, a0, a1, 0u, 0u, tiles[(2 * kt + 1) * 32 + lane]);
+        act(d0, A[kt][0], A[kt][1]);
+        act(d1, A[kt][2], A[kt][3]);
+    }
+    // layers 2 and 3 streamed: each pair of layer-2 N tiles is one K tile of
+    // layer 3, consumed as soon as it is formed
+    const uint2 *t2 = tiles + kTilesL1 * 32;
+    const uint2 *t3 = tiles + (kTilesL1 + kTilesL2) * 32;
+    const float2 c3 = *reinterpret_cast<const float2 *>(b3 + 2 * t);
+    d3[0] = c3.x; d3[1] = c3.y; d3[2] = c3.x; d3[3] = c3.y;
+#pragma unroll
+    for (int k3 = 0; k3 < 4; ++k3) {
+        const float2 c0 = *reinterpret_cast<const float2 *>(b2 + 16 * k3 + 2 * t);
+        const float2 c1 = *reinterpret_cast<const float2 *>(b2 + 16 * k3 + 8 + 2 * t);
+        float e0[4] = {c0.x, c0.y, c0.x, c0.y}, e1[4] = {c1.x, c1.y, c1.x, c1.y};
+#pragma unroll
+        for (int kt = 0; kt < 4; ++kt) {
+            mma_bf16_16816(e0, A[kt][0], A[kt][1], A[kt][2], A[kt][3], t2[((2 * k3) * 4 + kt) * 32 + lane]);
+            mma_bf16_16816(e1, A[kt][0], A[kt][1], A[kt][2], A[kt][3], t2[((2 * k3 + 1) * 4 + kt) * 32 + lane]);
+        }
+        uint32_t h0, h1, h2, h3;
+        act(e0, h0, h1);
+        act(e1, h2, h3);
+        mma_bf16_16816(d3, h0, h1, h2, h3, t3[k3 * 32 + lane]);
+    }
+}
+
 // MLP outputs (o1, o2) of this lane's trajectory; all 32 lanes must call.
 // `tiles` / `bias` may point to shared or global memory. want: the lanes whose
-// outputs are needed; an M tile without any is left out (a tail warp with its
-// live lanes in one half). Both M tiles at once, sharing the weight loads, cost
-// 64-300 bytes of spills and were no faster (30.8 against 30.6 ms on 2^18 paths).
+// outputs are needed. Up to eight of them (a warp of the launch's tail) share
+// the first eight rows of one tile, a quarter of the activations; else an M tile
+// (lanes 0-15, 16-31) without any is left out. A row's sums do not depend on the
+// other rows, so the outputs are the same. Both M tiles at once, sharing the
+// weight loads, cost 64-300 bytes of spills and were no faster (30.8 against
+// 30.6 ms on 2^18 paths).
 __device__ __forceinline__ void mlp_forward_warp(const uint2 *tiles, const float *bias, float in0,
                                                  float in1, float in2, unsigned want, float &o1, float &o2)
 {
     const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const float *b1 = bias, *b2 = bias + kMlpH, *b3 = bias + 2 * kMlpH;
+    const int lane = threadIdx.x & 31, g = lane >> 2;
     o1 = 0.0f;
     o2 = 0.0f;
+    float d3[4];
+    if (__popc(want) <= 8) {
+        int src = 0;                     // lane of the g-th wanted state
+        unsigned m = want;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            if (g == i && m) src = __ffs(m) - 1;
+            m &= m - 1u;
+        }
+        mlp_tile<true>(tiles, bias, in0, in1, in2, src, src, d3);
+        const int at = 4 * (__popc(want & ((1u << lane) - 1u)) & 7);
+        o1 = __shfl_sync(FULL, d3[0], at);
+        o2 = __shfl_sync(FULL, d3[1], at);
+        return;
+    }
 #pragma unroll 1
     for (int m = 0; m < 2; ++m) {
         if (!((want >> (16 * m)) & 0xffffu)) continue;
-        const int r0 = 16 * m + g, r1 = r0 + 8;
-        const float x0 = __shfl_sync(FULL, in0, r0), y0 = __shfl_sync(FULL, in1, r0), z0 = __shfl_sync(FULL, in2, r0);
-        const float x1 = __shfl_sync(FULL, in0, r1), y1 = __shfl_sync(FULL, in1, r1), z1 = __shfl_sync(FULL, in2, r1);
-        // layer-1 A fragment: row r, columns (2t, 2t+1) of (s0, s1, s2, 0, ..., 0)
-        const uint32_t a0 = pack_bf16x2(t == 0 ? x0 : (t == 1 ? z0 : 0.0f), t == 0 ? y0 : 0.0f);
-        const uint32_t a1 = pack_bf16x2(t == 0 ? x1 : (t == 1 ? z1 : 0.0f), t == 0 ? y1 : 0.0f);
-        // layer 1, two N tiles at a time -> the four K tiles of layer 2's A operand
-        uint32_t A[4][4];
-#pragma unroll
-        for (int kt = 0; kt < 4; ++kt) {
-            float d0[4], d1[4];
-            const float2 c0 = *reinterpret_cast<const float2 *>(b1 + 16 * kt + 2 * t);
-            const float2 c1 = *reinterpret_cast<const float2 *>(b1 + 16 * kt + 8 + 2 * t);
-            d0[0] = c0.x; d0[1] = c0.y; d0[2] = c0.x; d0[3] = c0.y;
-            d1[0] = c1.x; d1[1] = c1.y; d1[2] = c1.x; d1[3] = c1.y;
-            mma_bf16_16816(d0, a0, a1, 0u, 0u, tiles[(2 * kt) * 32 + lane]);
-            mma_bf16_16816(d1, a0, a1, 0u, 0u, tiles[(2 * kt + 1) * 32 + lane]);
-            A[kt][0] = pack_bf16x2(silu_f(d0[0]), silu_f(d0[1]));
-            A[kt][1] = pack_bf16x2(silu_f(d0[2]), silu_f(d0[3]));
-            A[kt][2] = pack_bf16x2(silu_f(d1[0]), silu_f(d1[1]));
-            A[kt][3] = pack_bf16x2(silu_f(d1[2]), silu_f(d1[3]));
-        }
-        // layers 2 and 3 streamed: each pair of layer-2 N tiles is one K tile of
-        // layer 3, consumed as soon as it is formed
-        const uint2 *t2 = tiles + kTilesL1 * 32;
-        const uint2 *t3 = tiles + (kTilesL1 + kTilesL2) * 32;
-        const float2 c3 = *reinterpret_cast<const float2 *>(b3 + 2 * t);
-        float d3[4] = {c3.x, c3.y, c3.x, c3.y};
-#pragma unroll
-        for (int k3 = 0; k3 < 4; ++k3) {
-            float e0[4], e1[4];
-            const float2 c0 = *reinterpret_cast<const float2 *>(b2 + 16 * k3 + 2 * t);
-            const float2 c1 = *reinterpret_cast<const float2 *>(b2 + 16 * k3 + 8 + 2 * t);
-            e0[0] = c0.x; e0[1] = c0.y; e0[2] = c0.x; e0[3] = c0.y;
-            e1[0] = c1.x; e1[1] = c1.y; e1[2] = c1.x; e1[3] = c1.y;
-#pragma unroll
-            for (int kt = 0; kt < 4; ++kt) {
-                mma_bf16_16816(e0, A[kt][0], A[kt][1], A[kt][2], A[kt][3], t2[((2 * k3) * 4 + kt) * 32 + lane]);
-                mma_bf16_16816(e1, A[kt][0], A[kt][1], A[kt][2], A[kt][3], t2[((2 * k3 + 1) * 4 + kt) * 32 + lane]);
-            }
-            const uint32_t h0 = pack_bf16x2(silu_f(e0[0]), silu_f(e0[1]));
-            const uint32_t h1 = pack_bf16x2(silu_f(e0[2]), silu_f(e0[3]));
-            const uint32_t h2 = pack_bf16x2(silu_f(e1[0]), silu_f(e1[1]));
-            const uint32_t h3 = pack_bf16x2(silu_f(e1[2]), silu_f(e1[3]));
-            mma_bf16_16816(d3, h0, h1, h2, h3, t3[k3 * 32 + lane]);
-        }
+        mlp_tile<false>(tiles, bias, in0, in1, in2, 16 * m + g, 16 * m + g + 8, d3);
         // lanes with t == 0 hold (o1, o2) of rows g (d3[0..1]) and g + 8 (d3[2..3])
         const int src = 4 * (lane & 7);
         const float s0 = __shfl_sync(FULL, d3[0], src), s1 = __shfl_sync(FULL, d3[1], src);
