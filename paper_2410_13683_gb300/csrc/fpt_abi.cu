@@ -120,6 +120,9 @@ struct fpt_ctx {
     long long tmp_cap = 0;
     // deterministic backward: per-block partial gradients, record order
     float *d_gpart = nullptr;
+    long long gpart_cap = 0;
+    double *d_accs = nullptr;
+    long long accs_cap = 0;
     uint32_t *d_perm = nullptr;
     long long perm_cap = 0;
     int *d_cnt = nullptr;
@@ -246,6 +249,7 @@ static void free_all(fpt_ctx *ctx)
     dev_free(ctx, ctx->d_grad);
     dev_free(ctx, ctx->d_tmp);
     dev_free(ctx, ctx->d_gpart);
+    dev_free(ctx, ctx->d_accs);
     dev_free(ctx, ctx->d_perm);
     dev_free(ctx, ctx->d_cnt);
     dev_free(ctx, ctx->d_off);
@@ -1392,12 +1396,33 @@ fpt_status fpt_mlp_pack(fpt_ctx *ctx, const float *params, void *blob, void *cud
     return FPT_OK;
 }
 
-// Per-block partial gradients of the backward (fixed size per device).
-static fpt_status ensure_gpart(fpt_ctx *ctx)
+// Per-block partial gradients of the backward (5.5 MB a network), for up to `nets`
+// networks in one launch; one where the context's memory is capped, fewer where
+// the device is full. *got: how many.
+static fpt_status ensure_gpart(fpt_ctx *ctx, int nets, int *got)
 {
-    if (ctx->d_gpart) return FPT_OK;
-    CK(dev_malloc(ctx, &ctx->d_gpart, sizeof(float) * (size_t)mlp_bwd_max_blocks(ctx->sm_count) * kMlpParams));
-    return FPT_OK;
+    int blocks = 0;
+    CK(mlp_bwd_blocks(ctx->sm_count, &blocks));
+    const long long per_net = (long long)blocks * kMlpParams;
+    for (nets = ctx->dev_limit ? 1 : std::min(nets, kTrainNets);; nets /= 2) {
+        const fpt_status st = ensure_dev(ctx, ctx->d_gpart, ctx->gpart_cap, nets * per_net);
+        if (st != FPT_E_NOMEM || nets == 1) {
+            *got = nets;
+            return st;
+        }
+        cudaGetLastError();   // the refused allocation
+    }
+}
+
+// One network that uses records [0, n) with the caller's output gradients.
+static TrainBatch direct_batch(long long n, float alpha_max)
+{
+    TrainBatch B;
+    std::memset(&B, 0, sizeof(B));
+    B.count = 1;
+    B.net[0].n_rec = n;
+    B.net[0].amax = alpha_max;
+    return B;
 }
 
 fpt_status fpt_mlp_eval(fpt_ctx *ctx, const void *blob, const float *s_in, const float *tan_t, int64_t n,
@@ -1440,13 +1465,15 @@ fpt_status fpt_mlp_grad(fpt_ctx *ctx, const float *params, const float *s_in, co
     }
     fpt_status st = ensure_dev(ctx, ctx->d_tmp, ctx->tmp_cap, 9 * n + 2 * kMlpParams);
     if (st != FPT_OK) return st;
-    if ((st = ensure_gpart(ctx)) != FPT_OK) return st;
+    int nets = 1;
+    if ((st = ensure_gpart(ctx, 1, &nets)) != FPT_OK) return st;
+    TrainBatch B = direct_batch(n, alpha_max);
     float *drec = ctx->d_tmp, *dd = drec + 8 * n, *dp = dd + n, *dg = dp + kMlpParams;
     CK(cudaMemcpyAsync(drec, hrec.data(), sizeof(float) * 8 * n, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(dd, hd.data(), sizeof(float) * n, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(dp, hp.data(), sizeof(float) * kMlpParams, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(dg, 0, sizeof(float) * kMlpParams, s));
-    CK(mlp_bwd_launch(dp, drec, n, nullptr, 0.0f, alpha_max, dd, dg, ctx->sm_count, s, nullptr, ctx->d_gpart));
+    CK(mlp_bwd_launch(B, dp, drec, n, nullptr, dd, dg, ctx->sm_count, s, nullptr, ctx->d_gpart));
     CK(cudaMemcpyAsync(grad, dg, sizeof(float) * kMlpParams, cudaMemcpyDefault, s));
     CK(cudaStreamSynchronize(s));
     return FPT_OK;
@@ -1470,13 +1497,15 @@ fpt_status fpt_mlp_grad2(fpt_ctx *ctx, const float *params, const float *s_in, c
     }
     fpt_status st = ensure_dev(ctx, ctx->d_tmp, ctx->tmp_cap, 10 * n + 2 * kMlpParams);
     if (st != FPT_OK) return st;
-    if ((st = ensure_gpart(ctx)) != FPT_OK) return st;
+    int nets = 1;
+    if ((st = ensure_gpart(ctx, 1, &nets)) != FPT_OK) return st;
+    TrainBatch B = direct_batch(n, alpha_max);
     float *drec = ctx->d_tmp, *dd = drec + 8 * n, *dp = dd + 2 * n, *dg = dp + kMlpParams;
     CK(cudaMemcpyAsync(drec, hrec.data(), sizeof(float) * 8 * n, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(dd, hd.data(), sizeof(float) * 2 * n, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(dp, hp.data(), sizeof(float) * kMlpParams, cudaMemcpyHostToDevice, s));
     CK(cudaMemsetAsync(dg, 0, sizeof(float) * kMlpParams, s));
-    CK(mlp_bwd_launch(dp, drec, n, nullptr, 0.0f, alpha_max, dd, dg, ctx->sm_count, s, nullptr, ctx->d_gpart, 1));
+    CK(mlp_bwd_launch(B, dp, drec, n, nullptr, dd, dg, ctx->sm_count, s, nullptr, ctx->d_gpart, 1));
     CK(cudaMemcpyAsync(grad, dg, sizeof(float) * kMlpParams, cudaMemcpyDefault, s));
     CK(cudaStreamSynchronize(s));
     return FPT_OK;
@@ -1560,7 +1589,8 @@ fpt_status fpt_mlp_train_round(fpt_ctx *ctx, const fpt_run_desc *run, int64_t ch
     if ((st = ensure_dev(ctx, ctx->d_perm, ctx->perm_cap, ctx->rec_cap)) != FPT_OK) return st;
     if ((st = ensure_dev(ctx, ctx->d_cnt, ctx->cnt_cap, ch)) != FPT_OK) return st;
     if ((st = ensure_dev(ctx, ctx->d_off, ctx->off_cap, ch)) != FPT_OK) return st;
-    if ((st = ensure_gpart(ctx)) != FPT_OK) return st;
+    int nets = 1;
+    if ((st = ensure_gpart(ctx, 1, &nets)) != FPT_OK) return st;
     CK(cudaMemsetAsync(ctx->d_grad, 0, sizeof(float) * kMlpParams, s));
     double sumY = 0, sumY2 = 0, sumN = 0;
     long long n_rec_total = 0, n_capped = 0, n_passed = 0;
@@ -1578,15 +1608,18 @@ fpt_status fpt_mlp_train_round(fpt_ctx *ctx, const fpt_run_desc *run, int64_t ch
         n_capped += ctx->h_flags[1];
         unsigned long long n_rec = 0;
         CK(cudaMemcpy(&n_rec, ctx->d_rec_cursor, sizeof(n_rec), cudaMemcpyDeviceToHost));
-        CK(mlp_coef_launch(ctx->d_nsteps, ctx->d_logw, sub.n_traj, m.dN, lambda, N_cut, 2.0 / (double)n_total,
-                           ctx->d_Y, ctx->d_acc, ctx->d_coef, s));
+        TrainBatch B;
+        std::memset(&B, 0, sizeof(B));
+        B.count = 1;
+        B.net[0] = TrainNet{0, sub.n_traj, 0, (long long)n_rec, m.dN, N_cut, 2.0 / (double)n_total,
+                            -sqrtf((float)m.dN), run->alpha_max, 0};
+        CK(mlp_coef_launch(B, ctx->d_nsteps, ctx->d_logw, lambda, ctx->d_Y, ctx->d_acc, ctx->d_coef, s));
         // records in a fixed order (by trajectory, then segment), so that the
         // gradient does not depend on the order the stepper appended them in
         CK(rec_order_launch(ctx->d_records, (long long)n_rec, sub.n_traj, run->mlp_segment, ctx->d_cnt,
                             ctx->d_off, ctx->d_perm, ctx->d_rec_err, s));
-        CK(mlp_bwd_launch(params, ctx->d_records, (long long)n_rec, ctx->d_coef, (float)m.dN, run->alpha_max,
-                          nullptr, ctx->d_grad, ctx->sm_count, s, ctx->d_perm, ctx->d_gpart,
-                          ctx->tables[run->model].rank2 ? 1 : 0));
+        CK(mlp_bwd_launch(B, params, ctx->d_records, (long long)n_rec, ctx->d_coef, nullptr, ctx->d_grad,
+                          ctx->sm_count, s, ctx->d_perm, ctx->d_gpart, ctx->tables[run->model].rank2 ? 1 : 0));
         double acc[2];
         int rec_err = 0;
         CK(cudaMemcpyAsync(acc, ctx->d_acc, sizeof(acc), cudaMemcpyDeviceToHost, s));
@@ -1677,10 +1710,9 @@ fpt_status fpt_mlp_train_batch(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n
     if ((st = ensure_dev(ctx, ctx->d_cnt, ctx->cnt_cap, total)) != FPT_OK) return st;
     if ((st = ensure_dev(ctx, ctx->d_off, ctx->off_cap, total)) != FPT_OK) return st;
     if ((st = ensure_dev(ctx, ctx->d_tmp, ctx->tmp_cap, (long long)n_runs * kMlpParams)) != FPT_OK) return st;
-    if ((st = ensure_gpart(ctx)) != FPT_OK) return st;
-    double *d_accs = nullptr;
-    CK(dev_malloc(ctx, &d_accs, sizeof(double) * acc_doubles * n_runs));
-    struct Free { fpt_ctx *c; double *p; ~Free() { dev_free(c, p); } } free_accs{ctx, d_accs};
+    int nets = 1;
+    if ((st = ensure_gpart(ctx, n_runs, &nets)) != FPT_OK) return st;
+    if ((st = ensure_dev(ctx, ctx->d_accs, ctx->accs_cap, (long long)(acc_doubles * n_runs))) != FPT_OK) return st;
 
     // one launch generates every run's paths with segment records
     ctx->record_mode = true;
@@ -1707,28 +1739,35 @@ fpt_status fpt_mlp_train_batch(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n
     if (rec_err) return fail(ctx, FPT_E_STATE, "segment records out of order (code " + std::to_string(rec_err) + ")");
     float *d_grads = ctx->d_tmp;
     CK(cudaMemsetAsync(d_grads, 0, sizeof(float) * (size_t)n_runs * kMlpParams, s));
-    for (int k = 0; k < n_runs; ++k) {
-        const fpt_run_desc &d = runs[k];
-        const fpt_model &m = ctx->models[d.model];
-        const long long b = begin[k], n = d.n_traj;
-        const long long r0 = off[b], r1 = (k + 1 < n_runs) ? off[begin[k + 1]] : (long long)n_rec;
-        // coefficients of run k's paths at their launch units (the backward indexes coef by unit)
-        CK(mlp_coef_launch(ctx->d_nsteps + b, ctx->d_logw + b, n, m.dN, lambda, N_cut[k], 2.0 / (double)n,
-                           ctx->d_Y + b, d_accs + (size_t)k * acc_doubles, ctx->d_coef + b, s));
-        CK(mlp_bwd_launch(params + (size_t)k * kMlpParams, ctx->d_records, r1 - r0, ctx->d_coef, (float)m.dN,
-                          d.alpha_max, nullptr, d_grads + (size_t)k * kMlpParams, ctx->sm_count, s,
-                          ctx->d_perm + r0, ctx->d_gpart, 0, (long long)n_rec));
-        CK(mlp_adam_launch(params + (size_t)k * kMlpParams, d_grads + (size_t)k * kMlpParams,
-                           adam_m + (size_t)k * kMlpParams, adam_v + (size_t)k * kMlpParams, kMlpParams, adam->lr,
-                           adam->beta1, adam->beta2, adam->eps, adam->step, adam->clip, s));
-        CK(mlp_pack_launch(params + (size_t)k * kMlpParams, static_cast<char *>(blobs) + (size_t)k * kMlpBlobBytes, s));
-        if (stats) {
-            stats[k].n_traj = n;
-            stats[k].n_records = r1 - r0;
+    // `nets` networks to a launch; a network's result does not depend on the others
+    for (int k0 = 0; k0 < n_runs; k0 += nets) {
+        TrainBatch B;
+        std::memset(&B, 0, sizeof(B));
+        B.count = std::min(nets, n_runs - k0);
+        for (int j = 0; j < B.count; ++j) {
+            const int k = k0 + j;
+            const fpt_run_desc &d = runs[k];
+            const fpt_model &m = ctx->models[d.model];
+            const long long b = begin[k];
+            const long long r0 = off[b], r1 = (k + 1 < n_runs) ? off[begin[k + 1]] : (long long)n_rec;
+            // coefficients at the launch units of the run's paths (the backward indexes coef by unit)
+            B.net[j] = TrainNet{b, d.n_traj, r0, r1 - r0, m.dN, N_cut[k], 2.0 / (double)d.n_traj,
+                                -sqrtf((float)m.dN), d.alpha_max, 0};
+            if (stats) {
+                stats[k].n_traj = d.n_traj;
+                stats[k].n_records = r1 - r0;
+            }
         }
+        CK(mlp_coef_launch(B, ctx->d_nsteps, ctx->d_logw, lambda, ctx->d_Y, ctx->d_accs + (size_t)k0 * acc_doubles,
+                           ctx->d_coef, s));
+        CK(mlp_bwd_launch(B, params + (size_t)k0 * kMlpParams, ctx->d_records, (long long)n_rec, ctx->d_coef, nullptr,
+                          d_grads + (size_t)k0 * kMlpParams, ctx->sm_count, s, ctx->d_perm, ctx->d_gpart, 0));
     }
+    CK(mlp_adam_launch(params, d_grads, adam_m, adam_v, n_runs * kMlpParams, adam->lr, adam->beta1, adam->beta2,
+                       adam->eps, adam->step, adam->clip, s));
+    CK(mlp_pack_launch(params, blobs, s, n_runs));
     std::vector<double> accs(acc_doubles * n_runs);
-    CK(cudaMemcpyAsync(accs.data(), d_accs, sizeof(double) * accs.size(), cudaMemcpyDeviceToHost, s));
+    CK(cudaMemcpyAsync(accs.data(), ctx->d_accs, sizeof(double) * accs.size(), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     if (stats) {
         for (int k = 0; k < n_runs; ++k) {

@@ -158,6 +158,24 @@ struct EmVariant {
     bool mnet;               // learned proposal with one network per run
 };
 
+// One network's share of a training step, and the networks of one launch.
+constexpr int kTrainNets = 16;
+struct TrainNet {
+    long long unit, n;         // first trajectory (launch unit) and their number
+    long long rec, n_rec;      // first record (in the record order) and their number
+    double dN, N_cut;
+    double scale;              // 2 / (trajectories of the whole round)
+    float neg_sqrt_dN, amax;
+    int blocks;                // backward: blocks of this network (set by mlp_bwd_launch)
+};
+struct TrainBatch {
+    int count, max_blocks;
+    TrainNet net[kTrainNets];
+};
+
+// Doubles of scratch of the loss coefficients, per network.
+__host__ __device__ constexpr size_t mlp_coef_scratch_doubles() { return 2 * 1024 + 2; }
+
 // Host wrappers implemented in fpt_kernels.cu.
 int em_occupancy(EmVariant v, int block, size_t smem_bytes);
 size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models, int pairs);
@@ -169,21 +187,19 @@ cudaError_t em_launch(const EmParams &p, EmVariant v, int grid, int block, size_
                       cudaStream_t s);
 
 // Host wrappers implemented in fpt_mlp.cu.
-cudaError_t mlp_pack_launch(const float *params, void *blob, cudaStream_t s);
+cudaError_t mlp_pack_launch(const float *params, void *blob, cudaStream_t s, int nets = 1);
 cudaError_t mlp_eval_launch(const void *blob, const float *s, const float *tan_t, long long n, float amax,
                             float *alpha, float *o, cudaStream_t st);
-cudaError_t mlp_coef_launch(const int32_t *nsteps, const double *logw, long long n, double dN, double lambda,
-                            double N_cut, double scale, double *Y, double *acc, float *coef, cudaStream_t s);
-cudaError_t mlp_bwd_launch(const float *params, const float *rec, long long n_rec, const float *coef, float dN,
-                           float amax, const float *dalpha_direct, float *grad, int sm_count, cudaStream_t s,
-                           const uint32_t *perm, float *partial, int rank2 = 0, long long rec_bound = 0);
-int mlp_bwd_max_blocks(int sm_count);
-size_t mlp_coef_scratch_doubles();
+cudaError_t mlp_coef_launch(const TrainBatch &B, const int32_t *nsteps, const double *logw, double lambda, double *Y,
+                            double *acc, float *coef, cudaStream_t s);
+cudaError_t mlp_bwd_launch(TrainBatch &B, const float *params, const float *rec, long long rec_bound, const float *coef,
+                           const float *dalpha_direct, float *grad, int sm_count, cudaStream_t s,
+                           const uint32_t *perm, float *partial, int rank2 = 0);
+cudaError_t mlp_bwd_blocks(int sm_count, int *blocks);
 cudaError_t rec_order_launch(const float *rec, long long n_rec, long long n_units, int segment, int *cnt,
                              long long *off, uint32_t *perm, int *err, cudaStream_t s);
 cudaError_t mlp_adam_launch(float *P, const float *G, float *m, float *v, int n, float lr, float b1, float b2,
                             float eps, int step, float clip, cudaStream_t s);
-size_t mlp_bwd_smem();
 cudaError_t hist_launch(const HistParams &p, double *out, cudaStream_t s);
 cudaError_t hist_noalloc_launch(HistParams p, double *out, cudaStream_t s);
 size_t hist_noalloc_scratch_bytes();

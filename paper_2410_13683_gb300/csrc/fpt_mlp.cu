@@ -32,8 +32,12 @@ __device__ __forceinline__ float w_kn(const float *P, int layer, int k, int n)
     return (n < kMlpOut) ? P[kOffW3 + n * kMlpH + k] : 0.0f;
 }
 
-__global__ void mlp_pack_kernel(const float *__restrict__ P, uint2 *__restrict__ tiles, float *__restrict__ bias)
+// Network blockIdx.y: parameters at P + y kMlpParams, blob at blob + y kMlpBlobBytes.
+__global__ void mlp_pack_kernel(const float *__restrict__ P, unsigned char *__restrict__ blob)
 {
+    P += (size_t)blockIdx.y * kMlpParams;
+    uint2 *tiles = reinterpret_cast<uint2 *>(blob + (size_t)blockIdx.y * kMlpBlobBytes);
+    float *bias = reinterpret_cast<float *>(tiles + kMlpTiles * 32);
     const int id = blockIdx.x * blockDim.x + threadIdx.x;
     if (id < kMlpTiles * 32) {
         const int tile = id >> 5, lane = id & 31, g = lane >> 2, t = lane & 3;
@@ -56,11 +60,10 @@ __global__ void mlp_pack_kernel(const float *__restrict__ P, uint2 *__restrict__
     }
 }
 
-cudaError_t mlp_pack_launch(const float *params, void *blob, cudaStream_t s)
+cudaError_t mlp_pack_launch(const float *params, void *blob, cudaStream_t s, int nets)
 {
-    uint2 *tiles = reinterpret_cast<uint2 *>(blob);
-    float *bias = reinterpret_cast<float *>(tiles + kMlpTiles * 32);
-    mlp_pack_kernel<<<(kMlpTiles * 32 + 255) / 256, 256, 0, s>>>(params, tiles, bias);
+    mlp_pack_kernel<<<dim3((kMlpTiles * 32 + 255) / 256, nets), 256, 0, s>>>(params,
+                                                                             static_cast<unsigned char *>(blob));
     return cudaGetLastError();
 }
 
@@ -103,21 +106,37 @@ cudaError_t mlp_eval_launch(const void *blob, const float *s, const float *tan_t
 // loss coefficients: c_j = (2/n)(Y_j - b), Y_j = ln w_j + lambda min(N_j, N_cut),
 // with b = mean Y over the run; also writes sum Y and sum Y^2 (loss monitor).
 // The sums are deterministic: each block reduces its grid-stride share in a
-// fixed order into its own partial, and one thread adds the partials in block
+// fixed order into its own partial, and one warp adds the partials in a fixed
 // order (no floating-point atomics, so the result does not depend on timing).
+//
+// The kernels of a training step take up to kTrainNets networks in one launch
+// (blockIdx.y), each on its own trajectories and records: a round of 64
+// networks had 64 x 7 launches of a few microseconds each.
 // ---------------------------------------------------------------------------
 constexpr int kYBlocks = 1024;
 
-__global__ void __launch_bounds__(256) mlp_y_kernel(const int32_t *__restrict__ nsteps,
-                                                    const double *__restrict__ logw, long long n, double dN,
-                                                    double lambda, double N_cut, double *__restrict__ Y,
-                                                    double *__restrict__ part)
+__host__ __device__ __forceinline__ int y_blocks(long long n)
+{
+    const long long b = (n + 255) / 256;
+    return (int)(b < 1 ? 1 : b > kYBlocks ? kYBlocks : b);
+}
+
+__global__ void __launch_bounds__(256) mlp_y_kernel(const __grid_constant__ TrainBatch B,
+                                                    const int32_t *__restrict__ nsteps,
+                                                    const double *__restrict__ logw, double lambda,
+                                                    double *__restrict__ Y, double *__restrict__ acc)
 {
     __shared__ double r1[8], r2[8];
+    const TrainNet &net = B.net[blockIdx.y];
+    const long long n = net.n;
+    const int blocks = y_blocks(n);
+    if ((int)blockIdx.x >= blocks) return;
+    nsteps += net.unit; logw += net.unit; Y += net.unit;
+    double *part = acc + blockIdx.y * mlp_coef_scratch_doubles() + 2;
     double s1 = 0.0, s2 = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const double N = (double)nsteps[i] * dN;
-        const double y = logw[i] + lambda * fmin(N, N_cut);
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)blocks * blockDim.x) {
+        const double N = (double)nsteps[i] * net.dN;
+        const double y = logw[i] + lambda * fmin(N, net.N_cut);
         Y[i] = y;
         s1 += y;
         s2 += y * y;
@@ -139,34 +158,46 @@ __global__ void __launch_bounds__(256) mlp_y_kernel(const int32_t *__restrict__ 
     }
 }
 
-__global__ void sum_partials_kernel(const double *__restrict__ part, int nb, double *__restrict__ acc)
+// One warp per network: lane l adds partials l, l + 32, ... and the lanes are
+// added pairwise (one thread adding 1,024 of them took 89 us, FP64 latency).
+__global__ void __launch_bounds__(32) sum_partials_kernel(const __grid_constant__ TrainBatch B, double *__restrict__ acc)
 {
+    acc += blockIdx.x * mlp_coef_scratch_doubles();
+    const double *part = acc + 2;
+    const int nb = y_blocks(B.net[blockIdx.x].n);
     double t1 = 0.0, t2 = 0.0;
-    for (int b = 0; b < nb; ++b) { t1 += part[2 * b]; t2 += part[2 * b + 1]; }
-    acc[0] = t1;
-    acc[1] = t2;
+    for (int b = threadIdx.x; b < nb; b += 32) { t1 += part[2 * b]; t2 += part[2 * b + 1]; }
+    for (int o = 16; o > 0; o >>= 1) {
+        t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+        t2 += __shfl_xor_sync(0xffffffffu, t2, o);
+    }
+    if (threadIdx.x == 0) {
+        acc[0] = t1;
+        acc[1] = t2;
+    }
 }
 
-__global__ void mlp_coef_kernel(const double *__restrict__ Y, long long n, const double *__restrict__ acc,
-                                double scale, float *__restrict__ coef)
+__global__ void __launch_bounds__(256) mlp_coef_kernel(const __grid_constant__ TrainBatch B, const double *__restrict__ Y,
+                                                       const double *__restrict__ acc, float *__restrict__ coef)
 {
-    const double mean = acc[0] / (double)n;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        coef[i] = (float)(scale * (Y[i] - mean));
+    const TrainNet &net = B.net[blockIdx.y];
+    const int blocks = y_blocks(net.n);
+    if ((int)blockIdx.x >= blocks) return;
+    const double mean = acc[blockIdx.y * mlp_coef_scratch_doubles()] / (double)net.n;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < net.n; i += (long long)blocks * blockDim.x)
+        coef[net.unit + i] = (float)(net.scale * (Y[net.unit + i] - mean));
 }
-
-size_t mlp_coef_scratch_doubles() { return 2 * kYBlocks + 2; }
 
 // coef_j = scale (Y_j - mean Y); scale = 2/n of the whole round. acc holds
-// 2 kYBlocks + 2 doubles: the block partials, then (sum Y, sum Y^2).
-cudaError_t mlp_coef_launch(const int32_t *nsteps, const double *logw, long long n, double dN, double lambda,
-                            double N_cut, double scale, double *Y, double *acc, float *coef, cudaStream_t s)
+// mlp_coef_scratch_doubles() per network: (sum Y, sum Y^2), then the block partials.
+cudaError_t mlp_coef_launch(const TrainBatch &B, const int32_t *nsteps, const double *logw, double lambda, double *Y,
+                            double *acc, float *coef, cudaStream_t s)
 {
-    const int grid = (int)std::min<long long>(kYBlocks, std::max<long long>(1, (n + 255) / 256));
-    double *part = acc + 2;
-    mlp_y_kernel<<<grid, 256, 0, s>>>(nsteps, logw, n, dN, lambda, N_cut, Y, part);
-    sum_partials_kernel<<<1, 1, 0, s>>>(part, grid, acc);
-    mlp_coef_kernel<<<grid, 256, 0, s>>>(Y, n, acc, scale, coef);
+    int grid = 1;
+    for (int k = 0; k < B.count; ++k) grid = std::max(grid, y_blocks(B.net[k].n));
+    mlp_y_kernel<<<dim3(grid, B.count), 256, 0, s>>>(B, nsteps, logw, lambda, Y, acc);
+    sum_partials_kernel<<<B.count, 32, 0, s>>>(B, acc);
+    mlp_coef_kernel<<<dim3(grid, B.count), 256, 0, s>>>(B, Y, acc, coef);
     return cudaGetLastError();
 }
 
@@ -321,12 +352,19 @@ __device__ __forceinline__ void st_bf16x2(__nv_bfloat16 *p, float lo, float hi)
 }
 
 __global__ void __launch_bounds__(kBwdWarps * 32)
-mlp_bwd_kernel(const float *__restrict__ P, const float *__restrict__ rec, long long n_rec, long long rec_bound,
-               const float *__restrict__ coef, float neg_sqrt_dN, float amax,
-               const float *__restrict__ dalpha_direct, const uint32_t *__restrict__ perm,
-               float *__restrict__ partial, int rank2)
+mlp_bwd_kernel(const __grid_constant__ TrainBatch B, const float *__restrict__ P, const float *__restrict__ rec,
+               long long rec_bound, const float *__restrict__ coef, const float *__restrict__ dalpha_direct,
+               const uint32_t *__restrict__ perm, float *__restrict__ partial, int rank2)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const TrainNet &net = B.net[blockIdx.y];
+    const long long n_rec = net.n_rec;
+    const float neg_sqrt_dN = net.neg_sqrt_dN, amax = net.amax;
+    const int blocks = net.blocks;
+    if ((int)blockIdx.x >= blocks) return;
+    P += (size_t)blockIdx.y * kMlpParams;
+    if (perm) perm += net.rec;
+    partial += ((size_t)blockIdx.y * B.max_blocks + blockIdx.x) * kMlpParams;
     BwdSmem &S = *reinterpret_cast<BwdSmem *>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
     const unsigned FULL = 0xffffffffu;
@@ -379,7 +417,7 @@ mlp_bwd_kernel(const float *__restrict__ P, const float *__restrict__ rec, long 
     for (int i = 0; i < 3; ++i) gW3[i][0] = gW3[i][1] = gW3[i][2] = gW3[i][3] = 0.0f;
 
     const long long n_tiles = (n_rec + kBwdRows - 1) / kBwdRows;
-    for (long long tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    for (long long tile = blockIdx.x; tile < n_tiles; tile += blocks) {
         // ---- load records of this tile
         if (tid < kBwdRows) {
             const long long slot = tile * kBwdRows + tid;
@@ -568,7 +606,7 @@ mlp_bwd_kernel(const float *__restrict__ P, const float *__restrict__ rec, long 
     // column tiles of W3), so plain stores fill the whole row and the partials
     // are summed later in block order
     const int m0 = 16 * warp;
-    float *grad = partial + (size_t)blockIdx.x * kMlpParams;
+    float *grad = partial;
 #pragma unroll
     for (int nt = 0; nt < 9; ++nt) {
 #pragma unroll
@@ -601,48 +639,62 @@ mlp_bwd_kernel(const float *__restrict__ P, const float *__restrict__ rec, long 
     }
 }
 
-size_t mlp_bwd_smem() { return sizeof(BwdSmem); }
-
 // grad[i] += sum over blocks b = 0, 1, ... of partial[b][i], in block order.
-__global__ void mlp_grad_reduce_kernel(const float *__restrict__ partial, int nb, float *__restrict__ grad)
+__global__ void __launch_bounds__(256) mlp_grad_reduce_kernel(const __grid_constant__ TrainBatch B,
+                                                              const float *__restrict__ partial,
+                                                              float *__restrict__ grad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= kMlpParams) return;
+    const int nb = B.net[blockIdx.y].blocks;
+    const float *q = partial + (size_t)blockIdx.y * B.max_blocks * kMlpParams + i;
     float t = 0.0f;
-    for (int b = 0; b < nb; ++b) t += partial[(size_t)b * kMlpParams + i];
-    grad[i] += t;
+#pragma unroll 16
+    for (int b = 0; b < nb; ++b) t += q[(size_t)b * kMlpParams];
+    grad[(size_t)blockIdx.y * kMlpParams + i] += t;
 }
 
-int mlp_bwd_max_blocks(int sm_count) { return 3 * sm_count; }
+// Blocks resident at once, the most a network's backward is split into.
+cudaError_t mlp_bwd_blocks(int sm_count, int *blocks)
+{
+    const size_t smem = sizeof(BwdSmem);
+    cudaError_t e = cudaFuncSetAttribute(mlp_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int per_sm = 0;
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_bwd_kernel, kBwdWarps * 32, smem);
+    *blocks = std::max(1, std::min(per_sm, 3)) * sm_count;
+    return e;
+}
 
 // The gradient of a call is deterministic: records in the order perm gives
 // (nullptr: buffer order), tiles statically assigned to blocks, per-block
-// partials (partial: mlp_bwd_max_blocks(sm_count) x kMlpParams floats) added
-// in block order. grad accumulates (+=). n_rec records are used (perm[0 ..
-// n_rec) when perm is given); rec_bound is the number of records in the buffer,
-// the bound of a valid perm entry (0: n_rec).
-cudaError_t mlp_bwd_launch(const float *params, const float *rec, long long n_rec, const float *coef, float dN,
-                           float amax, const float *dalpha_direct, float *grad, int sm_count, cudaStream_t s,
-                           const uint32_t *perm, float *partial, int rank2, long long rec_bound)
+// partials (partial: count x mlp_bwd_blocks x kMlpParams floats) added
+// in block order. grad accumulates (+=). A network uses perm[rec .. rec + n_rec)
+// (records [0, n_rec) without perm); rec_bound is the number of records in the
+// buffer, the bound of a valid perm entry. Parameters and gradients of the
+// networks lie one after the other. A network's records are split over as many
+// blocks as are resident at once (registers allow two per SM), so the tile
+// partition, and with it the gradient, is fixed for a given device and does not
+// depend on the networks that share the launch.
+cudaError_t mlp_bwd_launch(TrainBatch &B, const float *params, const float *rec, long long rec_bound, const float *coef,
+                           const float *dalpha_direct, float *grad, int sm_count, cudaStream_t s,
+                           const uint32_t *perm, float *partial, int rank2)
 {
-    if (rec_bound <= 0) rec_bound = n_rec;
-    const size_t smem = sizeof(BwdSmem);
-    cudaError_t e = cudaFuncSetAttribute(mlp_bwd_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int most = 0;
+    cudaError_t e = mlp_bwd_blocks(sm_count, &most);
     if (e != cudaSuccess) return e;
-    if (n_rec <= 0) return cudaSuccess;
-    // one wave: as many blocks as are resident at once (registers allow two per
-    // SM), so no block waits for a second wave; the tile partition, and with it
-    // the gradient, is fixed for a given device
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mlp_bwd_kernel, kBwdWarps * 32, smem)))
-        return e;
-    per_sm = std::max(1, std::min(per_sm, 3));
-    const long long tiles = (n_rec + kBwdRows - 1) / kBwdRows;
-    const int grid = (int)std::min<long long>(tiles, (long long)per_sm * sm_count);
-    mlp_bwd_kernel<<<grid, kBwdWarps * 32, smem, s>>>(params, rec, n_rec, rec_bound, coef, -sqrtf(dN), amax,
-                                                      dalpha_direct, perm, partial, rank2);
+    int grid = 0;
+    for (int k = 0; k < B.count; ++k) {
+        const long long tiles = (B.net[k].n_rec + kBwdRows - 1) / kBwdRows;
+        B.net[k].blocks = (int)std::min<long long>(tiles, most);
+        grid = std::max(grid, B.net[k].blocks);
+    }
+    if (grid == 0) return cudaSuccess;
+    B.max_blocks = most;
+    mlp_bwd_kernel<<<dim3(grid, B.count), kBwdWarps * 32, sizeof(BwdSmem), s>>>(B, params, rec, rec_bound, coef,
+                                                                               dalpha_direct, perm, partial, rank2);
     if ((e = cudaGetLastError())) return e;
-    mlp_grad_reduce_kernel<<<(kMlpParams + 255) / 256, 256, 0, s>>>(partial, grid, grad);
+    mlp_grad_reduce_kernel<<<dim3((kMlpParams + 255) / 256, B.count), 256, 0, s>>>(B, partial, grad);
     return cudaGetLastError();
 }
 
