@@ -1019,8 +1019,29 @@ __device__ __forceinline__ void run_group(const EmParams &P, Lane &L, bool &live
     ++L.grp;
 }
 
-// The same with a branch per step, for the interval in which a lane of the warp
-// reaches the step cap inside a group.
+// A group of an interval that is tried without looking for passages: the steps, the
+// weights and the noise sums only. Returns whether the lane's field was at or
+// below the end surface after one of the steps.
+template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
+__device__ __forceinline__ bool try_group(const EmParams &P, Lane &L, SegRec &sg, const float *z,
+                                          const float4 *__restrict__ tab, const ModelDev *s_model)
+{
+    const int n0 = 4 * L.grp;
+    float lw = 0.0f;
+    bool hit = false;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        any_step<WEIGHTED, SMEM, NIDX, DTAB, RANK2>(L, n0 + s, s, z, lw, tab, s_model, P.m0);
+        hit |= passed(L);
+    }
+    if (REC) add_xi<RANK2>(sg, z, 3);
+    if (WEIGHTED && lw != 0.0f) kahan_add(L.lw_hi, L.lw_lo, lw);
+    ++L.grp;
+    return hit;
+}
+
+// The same as run_group with a branch per step, for the interval in which a lane of
+// the warp reaches the step cap inside a group.
 template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
 __device__ __forceinline__ void run_group_guarded(const EmParams &P, Lane &L, bool &live, SegRec &sg,
                                                   const float *z, const float4 *__restrict__ tab,
@@ -1069,10 +1090,40 @@ __device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &l
     }
     const int nmax = SMEM ? P.m0.max_steps : L.nmax;
     const bool capped_inside = __any_sync(FULL, live && 4 * (L.grp + P.groups_per_check) > nmax);
-    float z[RANK2 ? 8 : 4];
+    constexpr int kZ = RANK2 ? 8 : 4;
+    float z[kZ];
     if (!capped_inside) {
-        for (int g = 0; g < P.groups_per_check; ++g) {
-            if (RING) ring.take(z);
+        bool again = true;
+        if (RING && MLP) {
+            // A lone warp waits for every group's passage test and branch. On the long
+            // paths of a learned proposal it tries the whole segment without them, and only
+            // if a live lane passed in it does it go back and take the segment again:
+            // training round of 2^15 paths 24.5 -> 22.7 ms, 2^18 learned paths 29.5 ->
+            // 28.6 ms. Where many short paths end in the tail the second attempts cost
+            // more than they give (16,384 linear paths 0.46 -> 0.50 ms), so the others
+            // look after every group.
+            const float x = L.x, x_c = L.x_c, p = L.p, p_c = L.p_c, lw_hi = L.lw_hi, lw_lo = L.lw_lo;
+            const float sx = sg.sum_xi, sy = sg.sum_xi2;
+            const int grp = L.grp;
+            bool hit = false;
+            float zn[kZ];
+            ring.take(zn);
+            for (int g = 1; g < P.groups_per_check; ++g) {
+#pragma unroll
+                for (int i = 0; i < kZ; ++i) z[i] = zn[i];
+                ring.take(zn);
+                hit |= try_group<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, sg, z, tab, s_model);
+            }
+            hit |= try_group<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, sg, zn, tab, s_model);
+            again = __any_sync(FULL, live && hit);
+            if (again) {
+                L.x = x; L.x_c = x_c; L.p = p; L.p_c = p_c; L.lw_hi = lw_hi; L.lw_lo = lw_lo;
+                sg.sum_xi = sx; sg.sum_xi2 = sy;
+                L.grp = grp;
+            }
+        }
+        for (int g = 0; again && g < P.groups_per_check; ++g) {
+            if (RING && !MLP) ring.take(z);
             else group_normals<RANK2>(P, L.rng, L.grp, z);
             run_group<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, z, tab, s_model);
         }
