@@ -83,6 +83,8 @@ struct fpt_ctx {
     uint8_t *d_status = nullptr;
     double *d_N = nullptr;
     long long unit_cap = 0;
+    float4 *d_parked = nullptr;         // two per path past its noise window
+    long long parked_cap = 0;
 
     // histogram scratch
     unsigned char *d_hist = nullptr;
@@ -239,6 +241,7 @@ static void free_all(fpt_ctx *ctx)
     dev_free(ctx, ctx->d_status);
     dev_free(ctx, ctx->d_N);
     dev_free(ctx, ctx->d_hist);
+    dev_free(ctx, ctx->d_parked);
     dev_free(ctx, ctx->d_hout);
     cudaFreeHost(ctx->h_hout);
     dev_free(ctx, ctx->d_records);
@@ -882,6 +885,29 @@ static fpt_status ensure_units(fpt_ctx *ctx, long long total)
     return FPT_OK;
 }
 
+// Buffer for the paths of a noise-window launch that outlive their window (32
+// bytes a path, 1 GB at most): none where the context's memory is capped or the
+// device is full, and the stepper then takes those steps itself.
+static long long ensure_parked(fpt_ctx *ctx, long long total)
+{
+    const long long want = std::min<long long>(total, 1LL << 25);
+    if (want <= ctx->parked_cap) return want;
+    if (ctx->dev_limit) return ctx->parked_cap;
+    if (ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
+    cudaStreamSynchronize(ctx->stream);
+    dev_free(ctx, ctx->d_parked);
+    ctx->d_parked = nullptr;
+    ctx->parked_cap = 0;
+    clear_graphs(ctx);
+    if (dev_malloc(ctx, &ctx->d_parked, sizeof(float4) * 2 * (size_t)want) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->d_parked = nullptr;
+        return 0;
+    }
+    ctx->parked_cap = want;
+    return want;
+}
+
 // Enqueue: descriptor upload, counter reset, status pre-fill, stepper launch,
 // flag read-back.
 static cudaError_t enqueue_run(fpt_ctx *ctx, const EmParams &p, EmVariant v, int grid,
@@ -1072,6 +1098,10 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
     p.sm_count = ctx->sm_count;
     p.pairs = pairs;
     p.mlp_run = mlp ? mlp_run : 0;
+    if (var.nidx && !var.rank2) {
+        p.park_cap = ensure_parked(ctx, total);
+        p.parked = ctx->d_parked;
+    }
     p.records = ctx->d_records;
     p.rec_cursor = ctx->d_rec_cursor;
     p.rec_cap = ctx->rec_cap;
@@ -1131,6 +1161,10 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
         } else {
             cudaError_t e = enqueue_run(ctx, p, var, grid, block, smem_bytes, n_runs, s);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "run launch");
+        }
+        if (p.park_cap) {
+            CK(classical_launch(p, ctx->sm_count, s));
+            CK(cudaMemcpyAsync(ctx->h_flags, ctx->d_flags, kFlagWords * sizeof(int), cudaMemcpyDeviceToHost, s));
         }
     } else {
         std::memset(ctx->h_flags, 0, kFlagWords * sizeof(int));

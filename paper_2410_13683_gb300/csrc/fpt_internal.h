@@ -116,7 +116,7 @@ struct EmParams {
     int smem_table_offset;     // SMEM mode: first entry of the staged table
     int smem_table_points;     // SMEM mode: entries staged
     long long total_units;
-    unsigned long long *cursor;
+    unsigned long long *cursor;   // units dealt, paths parked, parked paths dealt
     int *flags;                // flag words (kFlag*)
     int32_t *nsteps;
     double *logw;
@@ -130,6 +130,9 @@ struct EmParams {
     unsigned long long *t0;          // first %globaltimer reading of the launch (0 before)
     // learned proposal (MLP variants): launch-wide proposal, from the first MLP run
     int mlp_run;               // index of a run carrying the proposal parameters
+    // paths past their noise window (noise-window variant)
+    float4 *parked;            // [park_cap][2]
+    long long park_cap;        // 0: not parked
     // segment records (record variant)
     float *records;            // [rec_cap][8]
     unsigned long long *rec_cursor;
@@ -180,6 +183,8 @@ __host__ __device__ constexpr size_t mlp_coef_scratch_doubles() { return 2 * 102
 int em_occupancy(EmVariant v, int block, size_t smem_bytes);
 size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models, int pairs);
 int em_max_pairs();
+// Finishes the paths that a noise-window stepper parked (stream order after it).
+cudaError_t classical_launch(const EmParams &p, int sm_count, cudaStream_t s);
 // FPT_CHECKS builds: read and clear the device error word of the bounds checks
 // (kCheck* bits; synchronous). Other builds return 0.
 cudaError_t checks_take(int *word);

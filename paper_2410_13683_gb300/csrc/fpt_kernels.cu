@@ -1070,6 +1070,119 @@ __device__ __forceinline__ void run_group_guarded(const EmParams &P, Lane &L, bo
     ++L.grp;
 }
 
+// ---------------------------------------------------------------------------
+// Past the noise window
+// ---------------------------------------------------------------------------
+// After the last step of its noise window a path is classical: no normals, no
+// table, no weight. Left among noisy lanes it would take their full steps (65
+// instructions for 16), and more than half of a path's steps lie there (window of
+// 4.9 e-folds, paths of 11.5). So a lane is parked when its window has ended --
+// state into a buffer, the lane free for the next path -- and classical_kernel
+// finishes the parked paths after the stepper, all lanes alike. 10^6 paths:
+// 25.2 -> 15.9 ms. A lane that finds the buffer full goes on in the stepper.
+// Parked path: (x, x_c, pi, unit), (ln w pair, steps / 4, -).
+__device__ __forceinline__ void park(const EmParams &P, Lane &L, bool &live)
+{
+    const bool ended = live && L.nidx && 4 * L.grp > L.win_hi;
+    const unsigned m = __ballot_sync(0xffffffffu, ended);
+    if (!m || !P.park_cap) return;
+    const unsigned lane = threadIdx.x & 31u;
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(P.cursor + 1, (unsigned long long)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (!ended) return;
+    const unsigned long long i = base + __popc(m & ((1u << lane) - 1u));
+    if (i < (unsigned long long)P.park_cap) {
+        P.parked[2 * i] = make_float4(L.x, L.x_c, L.p, __uint_as_float(L.unit));
+        P.parked[2 * i + 1] = make_float4(L.lw_hi, L.lw_lo, __int_as_float(L.grp), 0.0f);
+        live = false;
+    } else {
+        L.win_hi = 0x7fffffff;           // every later step stays classical: the window has
+        L.win_lo = 0x7fffffff;           // not begun for it
+    }
+}
+
+// One classical step: em_step with S = T = 0 and no bias.
+__device__ __forceinline__ void classical_step(Lane &L, const ModelDev *s_model)
+{
+    const float vpv = drift_vpv<false, false>(L, nullptr, s_model, s_model[0]);
+    const float hdN = hh_dN<false>(L, s_model[0]);
+    const float dx = L.p * L.dN;
+    L.p = fmaf(hdN, L.p + vpv, L.p);
+    kahan_add(L.x, L.x_c, dx);
+}
+
+constexpr int kClassicalBlock = 256;
+
+__device__ __forceinline__ bool load_parked(const EmParams &P, Lane &L, unsigned long long i, unsigned long long count,
+                                            const RunSm *s_run, const ModelDev *s_model, unsigned &slot)
+{
+    if (i >= count) return false;
+    const float4 a = P.parked[2 * i];
+    lane_load(L, (long long)__float_as_uint(a.w), s_run, s_model, P.n_runs, P.rk);
+    L.x = a.x; L.x_c = a.y; L.p = a.z;
+    L.grp = __float_as_int(P.parked[2 * i + 1].z);
+    slot = (unsigned)i;
+    return true;
+}
+
+__global__ void __launch_bounds__(kClassicalBlock, 5) classical_kernel(const EmParams P)
+{
+    extern __shared__ __align__(16) float4 s_tab[];
+    __shared__ unsigned long long s_t0;
+    RunSm *s_run = smem_runs(s_tab, 0, false);
+    ModelDev *s_model = smem_models(s_run, P.n_runs);
+    const unsigned long long count = min(P.cursor[1], (unsigned long long)P.park_cap);
+    if (!count) return;
+    stage_launch<false, false>(P, s_tab, s_run, s_model, s_t0, nullptr);
+    const unsigned FULL = 0xffffffffu, lane = threadIdx.x & 31u;
+    Lane L{};
+    unsigned slot = 0;
+    const unsigned long long first = ((unsigned long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + lane;
+    bool live = load_parked(P, L, first, count, s_run, s_model, slot);
+    const unsigned long long dealt = (unsigned long long)gridDim.x * blockDim.x;
+
+    auto end = [&](int n, bool pas) {
+        const float4 w = P.parked[2 * (size_t)slot + 1];
+        L.lw_hi = w.x;
+        L.lw_lo = w.y;
+        finish(P, L, n, pas);
+        live = false;
+    };
+    while (__any_sync(FULL, live)) {
+        for (int g = 0; g < P.groups_per_check; ++g) {
+            bool h[4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                classical_step(L, s_model);
+                h[s] = passed(L);
+            }
+            const int n0 = 4 * L.grp;
+            if (live && ((h[0] | h[1] | h[2] | h[3]) || n0 + 4 >= L.nmax)) {
+                const int k = h[0] ? 0 : h[1] ? 1 : h[2] ? 2 : h[3] ? 3 : 4;
+                if (k < 4 && n0 + k + 1 <= L.nmax) end(n0 + k + 1, true);
+                else end(L.nmax, false);
+            }
+            ++L.grp;
+        }
+        const unsigned idle = __ballot_sync(FULL, !live);
+        if (idle) {
+            unsigned long long base = 0;
+            if (lane == 0) base = atomicAdd(P.cursor + 2, (unsigned long long)__popc(idle));
+            base = __shfl_sync(FULL, base, 0) + dealt;
+            if (!live) live = load_parked(P, L, base + __popc(idle & ((1u << lane) - 1u)), count, s_run, s_model, slot);
+        }
+        if (P.budget_ns && past_deadline(P, s_t0)) break;
+    }
+}
+
+cudaError_t classical_launch(const EmParams &p, int sm_count, cudaStream_t s)
+{
+    const size_t smem = em_smem_bytes(EmVariant{}, 0, p.n_runs, p.n_models, 0);
+    classical_kernel<<<5 * sm_count, kClassicalBlock, smem, s>>>(p);
+    return cudaGetLastError();
+}
+
 // One interval of the warp: the proposal's evaluation, the groups, the records.
 template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET, bool RANK2, bool RING>
 __device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &live, SegRec &sg, Ring<RANK2> &ring,
@@ -1138,6 +1251,7 @@ __device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &l
             run_group_guarded<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, z, tab, s_model);
         }
     }
+    if (NIDX) park(P, L, live);
     if (REC) write_records<RANK2>(P, L, sg);
 }
 

@@ -66,3 +66,22 @@ def test_every_path_runs_once_at_the_edges_of_a_launch(n):
         for x, y in zip(a, b):
             np.testing.assert_array_equal(x, y)
         assert (a[0] > 0).all() and (a[2] != fpt.FPT_TRAJ_ABORTED).all()
+
+
+@pytest.mark.parametrize("cap", [1 << 16, 4099])
+def test_paths_past_their_window_end_alike_with_and_without_the_buffer(cap):
+    """Paths that outlive their noise window are finished by a kernel of their own; where the context's memory
+    is capped the stepper takes those steps itself. Bit for bit, beside a run whose window never ends."""
+    S, Z = np.full(16, W.BM_S), np.zeros(16)
+    got = []
+    for capped in (False, True):
+        models = [replace(W.BM.model, max_steps=cap)] * 2
+        with fpt.fpt_init_model(models) as ctx:
+            fpt.fpt_noise_table(ctx, 0, fpt.FPT_TABLE_USER_N, 16, 1.0, 0.0, 3.9, S, Z)
+            fpt.fpt_noise_table(ctx, 1, fpt.FPT_TABLE_USER_N, 16, 1.0, 0.5, 90.0, S, Z)
+            if capped:
+                fpt.fpt_set_memory_limit(ctx, 4 << 30)
+            got.append(_run(ctx, [fpt.run_desc(0, 3001, seed=5, A=0.7),
+                                  fpt.run_desc(1, 1501, seed=5, run_id=1, A=0.7)]))
+    for a, b in zip(*got):
+        np.testing.assert_array_equal(a, b)
