@@ -147,6 +147,7 @@ struct HistParams {
     long long n;               // trajectories of the run
     double dN;
     double N_lo, db, N_tail;   // N_tail NaN: no tail set
+    double inv_dN;             // 1/dN (a first guess only)
     int n_bins;
     long long chunk;           // units per CTA of the summing kernel
     unsigned char *scratch;    // hist_scratch_bytes(n_bins) bytes, 64-byte aligned

@@ -1488,24 +1488,25 @@ __device__ __forceinline__ long long jk_begin(long long g, long long n)
     return (g * n + kJackknife - 1) / kJackknife;
 }
 
-// Smallest step count n in [-2^31, 2^31] with f(n) >= b, f nondecreasing (2^31:
-// none): bisection from a bracket around the guess g.
+// Smallest step count n in [-2^31, 2^31] that has reached a bound (2^31: none),
+// `reached` being false below it and true from it on: bisection from a bracket
+// around the guess g.
 template <class F>
-__device__ __forceinline__ long long first_n(double g, double b, F f)
+__device__ __forceinline__ long long first_n(double g, F reached)
 {
     const long long kMin = -2147483648LL, kEnd = 2147483648LL;
     long long lo = kMin - 1, hi = kEnd;
     const long long c = g >= (double)kEnd ? kEnd : (g > (double)kMin ? (long long)g : kMin);
     const long long p = max(c - 2, kMin), q = min(c + 2, kEnd - 1);
     if (p < kEnd) {
-        if (f(p) >= b) hi = p; else lo = p;
+        if (reached(p)) hi = p; else lo = p;
     }
     if (q > lo && q < hi) {
-        if (f(q) >= b) hi = q; else lo = q;
+        if (reached(q)) hi = q; else lo = q;
     }
     while (hi - lo > 1) {
         const long long m = lo + ((hi - lo) >> 1);
-        if (f(m) >= b) hi = m; else lo = m;
+        if (reached(m)) hi = m; else lo = m;
     }
     return hi;
 }
@@ -1533,7 +1534,16 @@ __global__ void __launch_bounds__(256) hist_prep_kernel(const HistParams P)
     // FP64 tasks spread over the blocks
     for (int j = (int)(threadIdx.x * gridDim.x + blockIdx.x); j < nb + 2 + 256; j += (int)nt) {
         if (j <= nb) {
-            const long long n = first_n((P.N_lo + (double)j * P.db) / P.dN, (double)j, q_of);
+            // q >= j: the division only where the product cannot tell (within 2^-48 of
+            // the bound; the quotient's own rounding is 2^-53), FP64 latency being what
+            // this kernel is made of
+            const double b = (double)j, at = b * P.db, sure = at * 3.6e-15;
+            const long long n = first_n((P.N_lo + at) * P.inv_dN, [&](long long m) {
+                const double x = __dsub_rn(N_of(m), P.N_lo), d = x - at;
+                if (j > 0 && d > sure) return true;
+                if (j > 0 && d < -sure) return false;
+                return __ddiv_rn(x, P.db) >= b;
+            });
             S.thr[j] = n;
             if (j == 0) {
                 // bins far narrower than a step: only the first step count can lie in range
@@ -1542,7 +1552,7 @@ __global__ void __launch_bounds__(256) hist_prep_kernel(const HistParams P)
                 S.head->off = n < 2147483648LL ? (float)q_of(n) : 0.0f;
             }
         } else if (j == nb + 1) {
-            S.head->n_tail = isnan(P.N_tail) ? 2147483648LL : first_n(P.N_tail / P.dN, P.N_tail, N_of);
+            S.head->n_tail = isnan(P.N_tail) ? 2147483648LL : first_n(P.N_tail * P.inv_dN, [&](long long m) { return N_of(m) >= P.N_tail; });
         } else {
             S.tab[j - nb - 2] = exp2((double)(j - nb - 2) * (1.0 / 256.0));
         }
@@ -1675,7 +1685,7 @@ __global__ void __launch_bounds__(kHistThreads) hist_sum_kernel(const HistParams
     __shared__ unsigned s_warp[kHistThreads / 32];
     const int nb = P.n_bins, nc = hist_classes(nb);
     const HistScratch S = hist_scratch(P.scratch, nb);
-    const bool smom = nc <= kHistSmemClasses;
+    const bool smom = nc <= kHistSmemClasses && P.chunk > kHistTile;   // a single tile adds to the totals at once
     double *s_tab = s_dynd, *s_M = s_tab + 256;
     long long *s_thr = reinterpret_cast<long long *>(s_M + nc);
     double *s_lw = reinterpret_cast<double *>(s_thr + nb + 1);
@@ -2018,12 +2028,12 @@ cudaError_t hist_launch(const HistParams &params, double *out, cudaStream_t s)
     cudaError_t e;
     hist_prep_kernel<<<64, 256, 0, s>>>(p);
     if ((e = cudaGetLastError())) return e;
-    // one block per SM and 1,024 paths at least
+    // short calls are latency: a block per 256 paths up to four per SM
     const size_t smax = 8 * ((size_t)nc + nb + 1);
     if (smax > 48 * 1024 &&
         (e = cudaFuncSetAttribute(hist_max_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax)))
         return e;
-    hist_max_kernel<<<(int)min(608LL, max(1LL, (p.n + 1023) / 1024)), 256, smax, s>>>(p);
+    hist_max_kernel<<<(int)min(608LL, max(1LL, (p.n + 255) / 256)), 256, smax, s>>>(p);
     if ((e = cudaGetLastError())) return e;
     // per jackknife block: CTAs of at least a tile
     const size_t ssum = hist_sum_smem(nb);
