@@ -122,8 +122,8 @@ __device__ __forceinline__ float sqrt_approx(float v)
 // 2^-22: neither is ever subnormal, so the flushing forms of the hardware
 // functions give the same bits without their subnormal handling, and -2 ln u0
 // is positive (all of this compared bit for bit over the 2^23 uniforms).
-// Executed instructions per step of direct sampling: 52.5; with the lane's Philox
-// products 38.1 -> 37.2 ms on 2^22 paths, noise window 26.1 -> 24.6 ms and
+// Executed instructions per step of direct sampling: 52.5, with the chained passage
+// test 50.8; with the lane's Philox products 38.1 -> 37.2 ms on 2^22 paths, noise window 26.1 -> 24.6 ms and
 // bump 10.6 -> 10.2 ms on 10^6.
 __device__ __forceinline__ float uniform23(uint32_t r)
 {
