@@ -1050,8 +1050,8 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
     const EmVariant var{weighted, smem, mlp, mlp && ctx->record_mode, nidx && !mlp, rank2 == 1, bump == 1,
                         mlp && mnet};
     const int entries = smem ? ctx->region_entries[smem_model] : 0, n_models = (int)ctx->models.size();
-    // the learned-proposal steppers are compiled for at most kMlpMaxBlock threads
-    const int block = mlp ? std::min(ctx->launch.block, kMlpMaxBlock) : ctx->launch.block;
+    // the learned-proposal steppers are compiled for smaller blocks
+    const int block = mlp ? std::min(ctx->launch.block, mnet ? kMnetMaxBlock : kMlpMaxBlock) : ctx->launch.block;
     // the helper warps' rings take shared memory that the blocks per SM leave free
     int pairs = em_max_pairs();
     const int occ_plain = em_occupancy(var, block, em_smem_bytes(var, entries, n_runs, n_models, 0));

@@ -40,6 +40,7 @@ constexpr int kMaxBins = 4096;
 constexpr int kNoAllocMaxBins = 1024;   // fpt_histogram_noalloc
 constexpr int kMlpHidden = 64;
 constexpr int kMlpMaxBlock = 384;       // block-size cap of the learned-proposal steppers
+constexpr int kMnetMaxBlock = 256;      // and of those with one network per run
 
 // Flag words of a stepper launch (64 bytes of device memory, zeroed before
 // the launch; the first kFlagWords ints are read back after it).

@@ -123,8 +123,8 @@ __device__ __forceinline__ float sqrt_approx(float v)
 // functions give the same bits without their subnormal handling, and -2 ln u0
 // is positive (all of this compared bit for bit over the 2^23 uniforms).
 // Executed instructions per step of direct sampling: 52.5, with the chained passage
-// test 50.8; with the lane's Philox products 38.1 -> 37.2 ms on 2^22 paths, noise window 26.1 -> 24.6 ms and
-// bump 10.6 -> 10.2 ms on 10^6.
+// test 50.8; with the lane's Philox products 38.1 -> 37.2 ms on 2^22 paths, noise
+// window 26.1 -> 24.6 ms and bump 10.6 -> 10.2 ms on 10^6.
 __device__ __forceinline__ float uniform23(uint32_t r)
 {
     return __uint_as_float(__funnelshift_r(r, 0x7fu, 9)) - 0.99999994039535522f;   // 1 - 2^-24
@@ -1265,11 +1265,15 @@ __device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &l
 }
 
 // Register budgets: two 512-thread blocks per SM (32 warps, at most 64
-// registers; direct sampling of 2^22 paths 46.1 ms with three blocks of 40
-// registers and guarded groups, 38.1 ms so); the learned-proposal steppers at most 384 threads per block and
-// two blocks, 80 registers: the network's fragments fit without spilling (a
-// 64-register build ran 512-thread blocks but executed ~7% more instructions
-// per step).
+// registers; three blocks of 40 registers: direct sampling of 2^22 paths 37.6 ms
+// against 36.0, eight biases 87.2 against 73.3); the learned-proposal steppers at
+// most 384 threads per block and two blocks, 80 registers: the network's
+// fragments fit without spilling (a 64-register build ran 512-thread blocks but
+// executed ~7% more instructions per step).
+// The steppers with one network per run keep each run's constants per lane and
+// take 256-thread blocks of 128 registers: of 80, 280-430 bytes were spilled
+// (training round of 64 networks x 1,024 paths 18.8 -> 18.3 ms, 64 x 8,192 paths
+// to a cap of 2^14 steps 15.7 -> 15.0 ms); the others gained nothing from it.
 template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET, bool RANK2>
 __device__ __forceinline__ void stepper(const EmParams &P)
 {
@@ -1329,7 +1333,7 @@ __device__ __forceinline__ void stepper(const EmParams &P)
 }
 
 template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET = false>
-__global__ void __launch_bounds__(MLP ? kMlpMaxBlock : 512, 2) em_kernel(const EmParams P)
+__global__ void __launch_bounds__(MNET ? kMnetMaxBlock : MLP ? kMlpMaxBlock : 512, 2) em_kernel(const EmParams P)
 {
     stepper<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, false>(P);
 }
