@@ -317,7 +317,7 @@ typedef struct {
 typedef struct {
     int32_t block;          /* threads per block: 128, 192, 256, 384 or 512
                                (default 512; learned-proposal launches use at
-                               most 384)                                      */
+                               most 384, with one network per run 256)        */
     int32_t blocks_per_sm;  /* resident blocks per SM (persistent grid)        */
     int32_t check_steps;    /* steps between refill points (multiple of 4)     */
     int32_t use_graph;      /* 1: replay a captured CUDA graph per shape; a
