@@ -766,8 +766,11 @@ __device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &l
     return true;
 }
 
+// bar.sync is the aligned form: all lanes of a warp must reach it together, and the
+// consumer comes to it from the divergent end of a group in which a lane passed.
 __device__ __forceinline__ void pair_barrier(int pair)
 {
+    __syncwarp();
     asm volatile("bar.sync %0, 64;" ::"r"(pair + 1) : "memory");
 }
 
