@@ -1306,7 +1306,9 @@ __device__ __forceinline__ void stepper(const EmParams &P)
     Ring<RANK2> ring{};
     // until the work is dealt out: an interval, then new trajectories for the idle lanes
     bool stop = false;
-    while (!*(volatile int *)&s_tail.dry) {
+    // (a vote: another warp may set dry between two lanes' reads, and all lanes must
+    // take part in the interval's warp-wide calls, or none)
+    while (!__any_sync(0xffffffffu, *(volatile int *)&s_tail.dry)) {
         run_interval<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, RANK2, false>(P, L, live, sg, ring, tab, s_run,
                                                                               s_model, s_tiles, s_bias, prun);
         refill_point(P, L, live, s_run, s_model, &s_tail.dry);
