@@ -17,6 +17,7 @@
 // N = n dN (Sec. 4.1).
 #include "fpt_internal.h"
 #include "fpt_mlp.cuh"
+#include "fpt_steps.h"
 
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -437,7 +438,7 @@ __device__ __forceinline__ void mlp_segment_start(Lane &L, bool live, SegRec &sg
         in0 = ((pr.mlp_flags & FPT_MLP_LOG_X) ? __logf(fmaxf(xv, pr.x_floor)) : xv);
         in0 = (in0 - pr.shift[0]) * pr.scale[0];
         in1 = (L.p - pr.shift[1]) * pr.scale[1];
-        in2 = ((float)(4 * L.grp) * dN - pr.shift[2]) * pr.scale[2];
+        in2 = ((float)steps_of(L.grp) * dN - pr.shift[2]) * pr.scale[2];
         float f;
         const float4 e = table_at<SMEM>(L, tab, f, M0);
         const float S = fmaf(f, e.y, e.x), T = fmaf(f, e.w, e.z);
@@ -453,7 +454,7 @@ __device__ __forceinline__ void mlp_segment_start(Lane &L, bool live, SegRec &sg
         if (REC) {
             sg.in0 = in0; sg.in1 = in1; sg.in2 = in2; sg.tan_t = tan_t; sg.raw = raw;
             sg.sum_xi = 0.0f;
-            sg.n0 = 4 * L.grp;
+            sg.n0 = steps_of(L.grp);
             sg.open = true;
         }
     }
@@ -482,7 +483,7 @@ __device__ __forceinline__ void mlp_segment_start_multi(Lane &L, bool live, SegR
             in0 = ((pr.mlp_flags & FPT_MLP_LOG_X) ? __logf(fmaxf(xv, pr.x_floor)) : xv);
             in0 = (in0 - pr.shift[0]) * pr.scale[0];
             in1 = (L.p - pr.shift[1]) * pr.scale[1];
-            in2 = ((float)(4 * L.grp) * dN - pr.shift[2]) * pr.scale[2];
+            in2 = ((float)steps_of(L.grp) * dN - pr.shift[2]) * pr.scale[2];
             float f;
             const float4 e = table_at<SMEM>(L, tab, f, M0);
             const float S = fmaf(f, e.y, e.x), T = fmaf(f, e.w, e.z);
@@ -500,7 +501,7 @@ __device__ __forceinline__ void mlp_segment_start_multi(Lane &L, bool live, SegR
             if (REC) {
                 sg.in0 = in0; sg.in1 = in1; sg.in2 = in2; sg.tan_t = tan_t; sg.raw = raw;
                 sg.sum_xi = 0.0f;
-                sg.n0 = 4 * L.grp;
+                sg.n0 = steps_of(L.grp);
                 sg.open = true;
             }
         }
@@ -875,7 +876,7 @@ __device__ __forceinline__ void mlp2_segment_start(Lane &L, bool live, SegRec &s
         in0 = ((pr.mlp_flags & FPT_MLP_LOG_X) ? __logf(fmaxf(xv, pr.x_floor)) : xv);
         in0 = (in0 - pr.shift[0]) * pr.scale[0];
         in1 = (L.p - pr.shift[1]) * pr.scale[1];
-        in2 = ((float)(4 * L.grp) * dN - pr.shift[2]) * pr.scale[2];
+        in2 = ((float)steps_of(L.grp) * dN - pr.shift[2]) * pr.scale[2];
     }
     float o1, o2;
     mlp_forward_warp(tiles, bias, in0, in1, in2, __ballot_sync(0xffffffffu, live), o1, o2);
@@ -889,7 +890,7 @@ __device__ __forceinline__ void mlp2_segment_start(Lane &L, bool live, SegRec &s
             sg.in0 = in0; sg.in1 = in1; sg.in2 = in2;
             sg.sum_xi = 0.0f;
             sg.sum_xi2 = 0.0f;
-            sg.n0 = 4 * L.grp;
+            sg.n0 = steps_of(L.grp);
             sg.open = true;
         }
     }
@@ -993,7 +994,7 @@ template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
 __device__ __forceinline__ void run_group(const EmParams &P, Lane &L, bool &live, SegRec &sg, const float *z,
                                           const float4 *__restrict__ tab, const ModelDev *s_model)
 {
-    const int n0 = 4 * L.grp;
+    const int n0 = steps_of(L.grp);
     float lw = 0.0f;
     // the fields after each step are kept for the lane that passed, the others have
     // one chained comparison a step (four flags instead: 64 models 32.0 ms
@@ -1038,7 +1039,7 @@ template <bool WEIGHTED, bool SMEM, bool REC, bool NIDX, bool DTAB, bool RANK2>
 __device__ __forceinline__ bool try_group(const EmParams &P, Lane &L, SegRec &sg, const float *z,
                                           const float4 *__restrict__ tab, const ModelDev *s_model)
 {
-    const int n0 = 4 * L.grp;
+    const int n0 = steps_of(L.grp);
     float lw = 0.0f;
     bool hit = false;
 #pragma unroll
@@ -1060,7 +1061,7 @@ __device__ __forceinline__ void run_group_guarded(const EmParams &P, Lane &L, bo
                                                   const ModelDev *s_model)
 {
     const int nmax = SMEM ? P.m0.max_steps : L.nmax;
-    int n = 4 * L.grp;
+    int n = steps_of(L.grp);
     float lw = 0.0f;
     bool done = !live;
 #pragma unroll
@@ -1095,7 +1096,7 @@ __device__ __forceinline__ void run_group_guarded(const EmParams &P, Lane &L, bo
 // Parked path: (x, x_c, pi, unit), (ln w pair, steps / 4, -).
 __device__ __forceinline__ void park(const EmParams &P, Lane &L, bool &live)
 {
-    const bool ended = live && L.nidx && 4 * L.grp > L.win_hi;
+    const bool ended = live && L.nidx && steps_of(L.grp) > L.win_hi;
     const unsigned m = __ballot_sync(0xffffffffu, ended);
     if (!m || !P.park_cap) return;
     const unsigned lane = threadIdx.x & 31u;
@@ -1169,10 +1170,10 @@ __global__ void __launch_bounds__(kClassicalBlock, 5) classical_kernel(const EmP
                 classical_step(L, s_model);
                 h[s] = passed(L);
             }
-            const int n0 = 4 * L.grp;
-            if (live && ((h[0] | h[1] | h[2] | h[3]) || n0 + 4 >= L.nmax)) {
+            const int n0 = steps_of(L.grp);
+            if (live && ((h[0] | h[1] | h[2] | h[3]) || cap_in_group(L.grp, L.nmax))) {
                 const int k = h[0] ? 0 : h[1] ? 1 : h[2] ? 2 : h[3] ? 3 : 4;
-                if (k < 4 && n0 + k + 1 <= L.nmax) end(n0 + k + 1, true);
+                if (k < 4 && step_within(L.grp, k, L.nmax)) end(n0 + k + 1, true);
                 else end(L.nmax, false);
             }
             ++L.grp;
@@ -1214,7 +1215,7 @@ __device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &l
         else mlp_segment_start<SMEM, REC>(L, live && L.mlp, sg, tab, s_tiles, s_bias, prun, P.m0);
     }
     const int nmax = SMEM ? P.m0.max_steps : L.nmax;
-    const bool capped_inside = __any_sync(FULL, live && 4 * (L.grp + P.groups_per_check) > nmax);
+    const bool capped_inside = __any_sync(FULL, live && cap_inside(L.grp, P.groups_per_check, nmax));
     constexpr int kZ = RANK2 ? 8 : 4;
     float z[kZ];
     if (!capped_inside) {
@@ -1252,8 +1253,8 @@ __device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &l
             else group_normals<RANK2>(P, L.rng, L.grp, z);
             run_group<WEIGHTED, SMEM, REC, NIDX, DTAB, RANK2>(P, L, live, sg, z, tab, s_model);
         }
-        if (live && 4 * L.grp >= nmax) {        // the cap falls on the interval's end
-            finish(P, L, 4 * L.grp, false);
+        if (live && cap_reached(L.grp, nmax)) {        // the cap falls on the interval's end
+            finish(P, L, steps_of(L.grp), false);
             live = false;
         }
     } else {
