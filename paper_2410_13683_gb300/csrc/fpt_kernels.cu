@@ -1492,6 +1492,12 @@ __device__ __forceinline__ double dkey_inv(unsigned long long k)
     return __longlong_as_double((long long)b);
 }
 
+// Reference of a class's deviations d = ln w - ref: its largest ln w, or 0 where that
+// is infinite (a class of zero weights, an infinite weight), so that the sums of d
+// are those of ln w itself. The sums of e = exp(ln w - M) of such a class mean
+// nothing; their values follow from M alone (hist_finalize_kernel).
+__device__ __forceinline__ double hist_ref(double M) { return isinf(M) ? 0.0 : M; }
+
 // Jackknife block g covers trajectories [ceil(g n / G), ceil((g+1) n / G)).
 __device__ __forceinline__ long long jk_begin(long long g, long long n)
 {
@@ -1710,7 +1716,7 @@ __global__ void __launch_bounds__(kHistThreads) hist_sum_kernel(const HistParams
     const unsigned FULL = 0xffffffffu;
 
     for (int i = tid; i < 256; i += kHistThreads) s_tab[i] = S.tab[i];
-    for (int i = tid; i < nc; i += kHistThreads) s_M[i] = S.key[i] ? dkey_inv(S.key[i]) : 0.0;
+    for (int i = tid; i < nc; i += kHistThreads) s_M[i] = S.key[i] ? hist_ref(dkey_inv(S.key[i])) : 0.0;
     if (smom)
         for (int i = tid; i < nc; i += kHistThreads) {
             for (int k = 0; k < 5; ++k) s_mom[5 * i + k] = 0.0;
@@ -1916,18 +1922,22 @@ __global__ void __launch_bounds__(128) hist_finalize_kernel(const HistParams P, 
         double cg = m[0], s1 = m[1], s2 = m[2], d1 = m[3], d2 = m[4];
         const unsigned long long key = S.key[b];
         double M = key ? dkey_inv(key) : 0.0;
+        if (isinf(M)) s1 = s2 = NAN;     // exp(M - M)
         unsigned long long kg, kt;
         hist_max_keys(S, nb, cut, any_tail, kg, kt);
         const double tc = warp_sum(cg), t1 = warp_sum(s1), t2 = warp_sum(s2);
-        // shares of this class in the sums over all weights and over the tail's
-        const bool in_tail = key && tail_class(b, cut, nb, any_tail);
+        // shares of this class in the sums over all weights and over the tail's: none
+        // where every weight is zero (a sum of ln w that is not a number has a weight
+        // that is none either)
+        const bool some = key && (M != -INFINITY || isnan(warp_sum(d1)));
+        const bool in_tail = some && tail_class(b, cut, nb, any_tail);
         {
-            const double x = on_lanes(key ? M - dkey_inv(kg) : 0.0, in_tail ? M - dkey_inv(kt) : 0.0, 0.0, 0.0);
+            const double x = on_lanes(some ? M - dkey_inv(kg) : 0.0, in_tail ? M - dkey_inv(kt) : 0.0, 0.0, 0.0);
             const double ex = exp(x), f = from_lane(ex, 0), h = from_lane(ex, 1);
             if (lane == 0) {
                 S.tot[5 * b] = tc;
-                S.tot[5 * b + 1] = f * t1;
-                S.tot[5 * b + 2] = f * S.swn[b];
+                S.tot[5 * b + 1] = some ? f * t1 : 0.0;
+                S.tot[5 * b + 2] = some ? f * S.swn[b] : 0.0;
                 S.tot[5 * b + 3] = in_tail ? h * t1 : 0.0;
                 S.tot[5 * b + 4] = in_tail ? h * h * t2 : 0.0;
             }
@@ -1938,18 +1948,25 @@ __global__ void __launch_bounds__(128) hist_finalize_kernel(const HistParams P, 
                 // the bin that the tail cuts: both parts about the larger of their maxima
                 const double *w = S.mom + ((size_t)lane * nc + nb + 2) * 5;
                 const double Mt = dkey_inv(S.key[nb + 2]), Ma = key ? M : Mt;
-                M = fmax(Ma, Mt);
-                const double da = Ma - M, dt = Mt - M, fa = exp(da), ft = exp(dt);
-                d2 = (d2 + 2.0 * da * d1 + cg * da * da) + (w[4] + 2.0 * dt * w[3] + w[0] * dt * dt);
+                M = dkey_inv(max(key, S.key[nb + 2]));
+                auto scale = [&](double Mp) { return Mp == M ? 1.0 : exp(Mp - M); };
+                auto part = [&](double Mp, double f, double v, double u) {
+                    return Mp == -INFINITY && Mp != M && !isnan(u) ? 0.0 : v * f;
+                };
+                const double fa = scale(Ma), ft = scale(Mt), none = isinf(Mt) ? NAN : 0.0;
+                s1 = part(Ma, fa, s1, d1) + part(Mt, ft, w[1] + none, w[3]);
+                s2 = part(Ma, fa * fa, s2, d1) + part(Mt, ft * ft, w[2] + none, w[3]);
+                // deviations about the common reference
+                const double da = hist_ref(Ma) - hist_ref(M), dt = hist_ref(Mt) - hist_ref(M);
+                auto shift2 = [](double c, double u, double u2, double h) { return isinf(u2) ? u2 : u2 + h * (2.0 * u + c * h); };
+                d2 = shift2(cg, d1, d2, da) + shift2(w[0], w[3], w[4], dt);
                 d1 = (d1 + cg * da) + (w[3] + w[0] * dt);
-                s1 = s1 * fa + w[1] * ft;
-                s2 = s2 * fa * fa + w[2] * ft * ft;
                 cg += w[0];
                 cnt = warp_sum(cg);
                 S1 = warp_sum(s1);
                 S2 = warp_sum(s2);
             }
-            const double D1 = warp_sum(d1), D2 = warp_sum(d2);
+            const double D1 = warp_sum(d1), D2 = warp_sum(d2), R = hist_ref(M);
             // delete-one-block jackknife of the weighted estimator
             const double ng = (double)(jk_begin(lane + 1, P.n) - jk_begin(lane, P.n));
             const double q = (S1 - s1) / (n - ng);
@@ -1971,14 +1988,14 @@ __global__ void __launch_bounds__(128) hist_finalize_kernel(const HistParams P, 
                                                 (kJackknife - 1.0) / kJackknife * ss));
                 const double lg = log(on_lanes(S1, S2, n * P.db));
                 const double lsw = M + from_lane(lg, 0);
-                const double ex = exp(on_lanes(lsw - from_lane(lg, 2), M, M + mean + 0.5 * v));
+                const double ex = exp(on_lanes(lsw - from_lane(lg, 2), M, R + mean + 0.5 * v));
                 const double eM = from_lane(ex, 1);
                 // per bin width: lognormal mean, errors of the weighted mean
                 const double r4 = on_lanes(share * from_lane(ex, 2), eM * from_lane(rt, 1), eM * from_lane(rt, 2)) / P.db;
                 const double pl = from_lane(r4, 0);
                 const bool two = cnt >= 2.0;
-                const double o[10] = {cnt, lsw, 2.0 * M + from_lane(lg, 1), D1 + cnt * M,
-                                      isinf(D2) ? D2 : D2 + M * (2.0 * D1 + cnt * M), from_lane(ex, 0),
+                const double o[10] = {cnt, lsw, 2.0 * M + from_lane(lg, 1), D1 + cnt * R,
+                                      isinf(D2) ? D2 : D2 + R * (2.0 * D1 + cnt * R), from_lane(ex, 0),
                                       from_lane(r4, 1), two ? pl : NAN, two ? pl * from_lane(rt, 0) : NAN,
                                       from_lane(r4, 2)};
                 if (lane == 0)
