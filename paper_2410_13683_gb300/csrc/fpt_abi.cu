@@ -1053,13 +1053,13 @@ fpt_status fpt_run(fpt_ctx *ctx, const fpt_run_desc *runs, int32_t n_runs, fpt_t
     // the learned-proposal steppers are compiled for smaller blocks
     const int block = mlp ? std::min(ctx->launch.block, mnet ? kMnetMaxBlock : kMlpMaxBlock) : ctx->launch.block;
     // the helper warps' rings take shared memory that the blocks per SM leave free
+    size_t most = 0;
+    CK(em_opt_in(var, &most));
+    auto smem_of = [&](int n_pairs) { return em_smem_bytes(var, entries, n_runs, n_models, n_pairs); };
+    const int occ = em_occupancy(var, block, smem_of(0), most);
     int pairs = em_max_pairs();
-    const int occ_plain = em_occupancy(var, block, em_smem_bytes(var, entries, n_runs, n_models, 0));
-    int occ = occ_plain;
-    while (pairs > 0 && (occ = em_occupancy(var, block, em_smem_bytes(var, entries, n_runs, n_models, pairs))) < occ_plain)
-        --pairs;
-    const size_t smem_bytes = em_smem_bytes(var, entries, n_runs, n_models, pairs);
-    if (pairs == 0) occ = em_occupancy(var, block, smem_bytes);   // the opt-in size of the launch
+    while (pairs > 0 && em_occupancy(var, block, smem_of(pairs), most) < occ) --pairs;
+    const size_t smem_bytes = smem_of(pairs);
     if (occ < 1) return fail(ctx, FPT_E_CUDA, "stepper does not fit on an SM with this shape");
     const int bps = ctx->launch.blocks_per_sm ? std::min(ctx->launch.blocks_per_sm, occ) : occ;
     // no more blocks than chunks of 32 trajectories: a block's first warp takes a chunk each

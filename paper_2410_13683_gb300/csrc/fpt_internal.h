@@ -182,7 +182,8 @@ struct TrainBatch {
 __host__ __device__ constexpr size_t mlp_coef_scratch_doubles() { return 2 * 1024 + 2; }
 
 // Host wrappers implemented in fpt_kernels.cu.
-int em_occupancy(EmVariant v, int block, size_t smem_bytes);
+cudaError_t em_opt_in(EmVariant v, size_t *most);
+int em_occupancy(EmVariant v, int block, size_t smem_bytes, size_t most);
 size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models, int pairs);
 int em_max_pairs();
 // Finishes the paths that a noise-window stepper parked (stream order after it).

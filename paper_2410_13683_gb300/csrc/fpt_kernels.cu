@@ -24,6 +24,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 
 namespace fpt_dev {
@@ -1400,20 +1401,36 @@ size_t em_smem_bytes(EmVariant v, int table_entries, int n_runs, int n_models, i
 
 int em_max_pairs() { return kMaxPairs; }
 
-// Opt in to the dynamic shared memory the table (and proposal) need, outside
-// any stream capture, then report resident blocks per SM for this shape.
-int em_occupancy(EmVariant v, int block, size_t smem_bytes)
+// Opt in to dynamic shared memory, outside any stream capture. The opt-in is state
+// of the kernel on the device, shared by every thread of the process, and a launch
+// above it is refused: it is always the most the kernel can have (*most), so that
+// contexts on other threads, which need other sizes, set the same value.
+cudaError_t em_opt_in(EmVariant v, size_t *most)
 {
     const void *f = em_fn(v);
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess)
-        return 0;
+    cudaFuncAttributes a;
+    cudaError_t e = cudaFuncGetAttributes(&a, f);
+    int dev = 0, bytes = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&bytes, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    bytes -= (int)a.sharedSizeBytes;
+    *most = (size_t)bytes;
+    return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+// Resident blocks per SM for this shape (0: it does not fit); most: from em_opt_in().
+int em_occupancy(EmVariant v, int block, size_t smem_bytes, size_t most)
+{
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f, block, smem_bytes) != cudaSuccess) return 0;
+    if (smem_bytes > most ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, em_fn(v), block, smem_bytes) != cudaSuccess)
+        return 0;
     return nb;
 }
 
-// Launch only (safe inside stream capture): em_occupancy() must have been
-// called for this shape first.
+// Launch only (safe inside stream capture): em_opt_in() must have been called for
+// this variant first.
 cudaError_t em_launch(const EmParams &p, EmVariant v, int grid, int block, size_t smem_bytes, cudaStream_t s)
 {
     void *args[] = {const_cast<EmParams *>(&p)};
@@ -2055,17 +2072,21 @@ cudaError_t hist_launch(const HistParams &params, double *out, cudaStream_t s)
     cudaError_t e;
     hist_prep_kernel<<<64, 256, 0, s>>>(p);
     if ((e = cudaGetLastError())) return e;
-    // short calls are latency: a block per 256 paths up to four per SM
-    const size_t smax = 8 * ((size_t)nc + nb + 1);
+    // short calls are latency: a block per 256 paths up to four per SM. The opt-in to
+    // more than 48 KB is shared by the threads of the process: every call sets the
+    // value of the largest histogram (see em_opt_in)
+    auto max_smem = [](int n) { return 8 * ((size_t)hist_classes(n) + n + 1); };
+    const size_t smax = max_smem(nb);
     if (smax > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(hist_max_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smax)))
+        (e = cudaFuncSetAttribute(hist_max_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem(kMaxBins))))
         return e;
     hist_max_kernel<<<(int)min(608LL, max(1LL, (p.n + 255) / 256)), 256, smax, s>>>(p);
     if ((e = cudaGetLastError())) return e;
     // per jackknife block: CTAs of at least a tile
     const size_t ssum = hist_sum_smem(nb);
+    const size_t ssum_most = std::max(hist_sum_smem(kMaxBins), hist_sum_smem(kHistSmemClasses - 3));
     if (ssum > 48 * 1024 &&
-        (e = cudaFuncSetAttribute(hist_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssum)))
+        (e = cudaFuncSetAttribute(hist_sum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ssum_most)))
         return e;
     const long long per_block = (p.n + kJackknife - 1) / kJackknife;
     const long long most = ssum > 113 * 1024 ? 4 : 9;             // one or two CTAs per SM: a single wave
