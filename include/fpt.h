@@ -550,7 +550,9 @@ fpt_status fpt_histogram_noalloc(const int32_t *nsteps, const double *logw, cons
  * FPT_E_NOMEM (fpt_last_error names the limit, the bytes in use and the bytes
  * requested), and the context stays usable -- a later call with a smaller
  * request, or after the limit is raised, succeeds. Memory already held is
- * kept. max_bytes = 0 removes the limit (the default); negative values are
+ * kept, except a buffer that only speeds up noise-window runs (32 bytes a
+ * path, at most 1 GB), which is given back where an allocation would be
+ * refused, by the limit or by the device. max_bytes = 0 removes the limit (the default); negative values are
  * FPT_E_INVALID. Serves memory budgeting beside other users of the GPU and
  * the injection of allocation failures.
  */

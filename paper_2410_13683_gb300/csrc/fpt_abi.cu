@@ -85,6 +85,8 @@ struct fpt_ctx {
     long long unit_cap = 0;
     float4 *d_parked = nullptr;         // two per path past its noise window
     long long parked_cap = 0;
+    long long parked_refused = 0;       // smallest size that was refused, and the calls
+    int parked_wait = 0;                // that still go without before it is asked for again
 
     // histogram scratch
     unsigned char *d_hist = nullptr;
@@ -182,17 +184,34 @@ static fpt_status take_checks(fpt_ctx *c)
 
 // Device allocations of a context: counted, and refused like an out-of-memory
 // cudaMalloc when they would take the context past its limit.
-template <class T>
-static cudaError_t dev_malloc(fpt_ctx *ctx, T **p, size_t bytes)
+static cudaError_t dev_malloc_once(fpt_ctx *ctx, void **p, size_t bytes)
 {
     if (ctx->dev_limit && ctx->dev_bytes + bytes > ctx->dev_limit) {
         ctx->refused_bytes = bytes;
         return cudaErrorMemoryAllocation;
     }
-    const cudaError_t e = cudaMalloc(reinterpret_cast<void **>(p), bytes);
-    if (e == cudaSuccess) {
-        ctx->dev_sizes[*p] = bytes;
-        ctx->dev_bytes += bytes;
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();             // not left for the check of a later launch
+        return e;
+    }
+    ctx->dev_sizes[*p] = bytes;
+    ctx->dev_bytes += bytes;
+    return e;
+}
+
+static void release_parked(fpt_ctx *ctx);
+
+// The buffer of parked paths only saves time: it is given back where another
+// allocation is refused.
+template <class T>
+static cudaError_t dev_malloc(fpt_ctx *ctx, T **p, size_t bytes)
+{
+    cudaError_t e = dev_malloc_once(ctx, reinterpret_cast<void **>(p), bytes);
+    if (e == cudaErrorMemoryAllocation && ctx->d_parked) {
+        release_parked(ctx);
+        ctx->refused_bytes = 0;
+        e = dev_malloc_once(ctx, reinterpret_cast<void **>(p), bytes);
     }
     return e;
 }
@@ -206,6 +225,17 @@ static void dev_free(fpt_ctx *ctx, void *p)
         ctx->dev_sizes.erase(it);
     }
     cudaFree(p);
+}
+
+// Graphs that hold the buffer's address get the call's parameters before they run.
+static void release_parked(fpt_ctx *ctx)
+{
+    if (!ctx->d_parked) return;
+    if (ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
+    cudaStreamSynchronize(ctx->stream);
+    dev_free(ctx, ctx->d_parked);
+    ctx->d_parked = nullptr;
+    ctx->parked_cap = 0;
 }
 
 #define CK(call)                                              \
@@ -887,24 +917,27 @@ static fpt_status ensure_units(fpt_ctx *ctx, long long total)
 
 // Buffer for the paths of a noise-window launch that outlive their window (32
 // bytes a path, 1 GB at most): none where the context's memory is capped or the
-// device is full, and the stepper then takes those steps itself.
+// device is full, and the stepper then takes those steps itself. A refused size is
+// asked for again after 64 calls, not on each.
 static long long ensure_parked(fpt_ctx *ctx, long long total)
 {
     const long long want = std::min<long long>(total, 1LL << 25);
     if (want <= ctx->parked_cap) return want;
     if (ctx->dev_limit) return ctx->parked_cap;
-    if (ctx->last_stream) cudaStreamSynchronize(ctx->last_stream);
-    cudaStreamSynchronize(ctx->stream);
-    dev_free(ctx, ctx->d_parked);
-    ctx->d_parked = nullptr;
-    ctx->parked_cap = 0;
-    clear_graphs(ctx);
-    if (dev_malloc(ctx, &ctx->d_parked, sizeof(float4) * 2 * (size_t)want) != cudaSuccess) {
-        cudaGetLastError();
-        ctx->d_parked = nullptr;
+    if (ctx->parked_wait > 0 && want >= ctx->parked_refused) {
+        --ctx->parked_wait;
+        return ctx->parked_cap;
+    }
+    release_parked(ctx);
+    void *p = nullptr;
+    if (dev_malloc_once(ctx, &p, sizeof(float4) * 2 * (size_t)want) != cudaSuccess) {
+        ctx->parked_refused = want;
+        ctx->parked_wait = 64;
         return 0;
     }
+    ctx->d_parked = static_cast<float4 *>(p);
     ctx->parked_cap = want;
+    ctx->parked_wait = 0;
     return want;
 }
 
