@@ -659,7 +659,7 @@ __device__ __forceinline__ bool refill_point(const EmParams &P, Lane &L, bool &l
 // Path lengths are heavy-tailed, so once the work cursor is dry the warps keep
 // one or two live lanes each for most of a launch, at the price of full ones.
 // From then on (tail mode) the warps of a block meet every tail_intervals
-// intervals (128 steps) and the live lanes of the last warps move into free
+// intervals (about 512 steps) and the live lanes of the last warps move into free
 // lanes of the first ones, through a small pool in shared memory, whenever that
 // empties a warp. A lane's state is eight words; everything else is loaded
 // from its run and model again. A lane moves between intervals, where no group
@@ -696,15 +696,16 @@ __device__ __forceinline__ int scan_incl(int v)
 }
 
 // One meeting of the block's warps. Returns false when the block has no live
-// lane left or must stop. kMinWarps: warps that compaction leaves busy if it can,
-// the lanes spread evenly over them. A warp with one network per run evaluates
-// the networks of its lanes in turn, so its lanes are spread over eight warps
-// (training round of 64 networks, 1,024 paths each: 26.7 ms with one, 24.4 with
-// two, 22.7 with eight); a step costs a warp the same for one lane and for 32,
-// so the others are better packed (2^18 learned paths: 30.3 ms with one, 33.2
-// with four, 47.7 with eight). Lane j of every warp holds the count of the warp at
-// position j, so all warps come to the same decision.
-template <int kMinWarps>
+// lane left or must stop. COMPACT: lanes move to as few warps as hold them; a step
+// costs a warp the same for one lane and for 32 (2^18 learned paths: 30.3 ms, with
+// four warps kept busy 33.2, with eight 47.7). Not in the steppers with one network
+// per run: a warp evaluates the networks of its lanes in turn, so lanes stay where
+// they are and only the helpers are handed out (training round of 64 networks,
+// 1,024 paths each, in blocks of eight warps: 18.8 ms; compacted to six warps 19.5,
+// four 19.9, two 21.5, one 22.8; 16 networks or 200 paths each: no difference).
+// Lane j of every warp holds the count of the warp at position j, so all warps come
+// to the same decision.
+template <bool COMPACT>
 __device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &live, bool stop, int round,
                                              TailSm &T, PairSm *pairs, const RunSm *s_run,
                                              const ModelDev *s_model, TailRole &role)
@@ -720,8 +721,8 @@ __device__ __forceinline__ bool tail_meeting(const EmParams &P, Lane &L, bool &l
     const int total = __reduce_add_sync(FULL, c);
     if (!total) return false;
     unsigned busy = __ballot_sync(FULL, c > 0);
-    const int need = max((total + 31) >> 5, min(kMinWarps, nw));
-    if (need < __popc(busy)) {
+    const int need = (total + 31) >> 5;
+    if (COMPACT && need < __popc(busy)) {
         // keep the first positions; the lanes of the later ones must fit the pool
         const int excl = scan_incl(c) - c;
         const unsigned fits = __ballot_sync(FULL, lane >= need && lane < nw && total - excl <= kPoolLanes);
@@ -1271,14 +1272,15 @@ __device__ __forceinline__ void run_interval(const EmParams &P, Lane &L, bool &l
 
 // Register budgets: two 512-thread blocks per SM (32 warps, at most 64
 // registers; three blocks of 40 registers: direct sampling of 2^22 paths 37.6 ms
-// against 36.0, eight biases 87.2 against 73.3); the learned-proposal steppers at
-// most 384 threads per block and two blocks, 80 registers: the network's
-// fragments fit without spilling (a 64-register build ran 512-thread blocks but
-// executed ~7% more instructions per step).
+// against 36.0, eight biases 87.2 against 73.3); spilled: nothing with the table in
+// shared memory, 12 bytes at most without. The learned-proposal steppers take at
+// most 384 threads per block and two blocks, 80 registers (a 64-register build ran
+// 512-thread blocks but executed ~7% more instructions per step); with the tail's
+// second copy of the interval they spill 20-82 bytes, with several models 76-226.
 // The steppers with one network per run keep each run's constants per lane and
-// take 256-thread blocks of 128 registers: of 80, 280-430 bytes were spilled
-// (training round of 64 networks x 1,024 paths 18.8 -> 18.3 ms, 64 x 8,192 paths
-// to a cap of 2^14 steps 15.7 -> 15.0 ms); the others gained nothing from it.
+// take 256-thread blocks of 128 registers: they spill 68-94 bytes, of 80 registers
+// 280-430 (training round of 64 networks x 1,024 paths 18.8 -> 18.3 ms, 64 x 8,192
+// paths to a cap of 2^14 steps 15.7 -> 15.0 ms); the others gained nothing from it.
 template <bool WEIGHTED, bool SMEM, bool MLP, bool REC, bool NIDX, bool DTAB, bool MNET, bool RANK2>
 __device__ __forceinline__ void stepper(const EmParams &P)
 {
@@ -1322,7 +1324,7 @@ __device__ __forceinline__ void stepper(const EmParams &P)
     // the tail
     TailRole role;
     for (int round = 0;
-         tail_meeting<MNET ? 8 : 1>(P, L, live, stop, round, s_tail, s_pairs, s_run, s_model, role); ++round) {
+         tail_meeting<!MNET>(P, L, live, stop, round, s_tail, s_pairs, s_run, s_model, role); ++round) {
         if (role.pair < 0) {
             for (int k = 0; k < P.tail_intervals; ++k)
                 run_interval<WEIGHTED, SMEM, MLP, REC, NIDX, DTAB, MNET, RANK2, false>(
