@@ -188,11 +188,12 @@ def roofline(steps_per_launch, launch_ms, sm_count, sm_max_mhz, traffic, instr_p
 
 def pipe_fractions(steps_per_s, sm_count, sm_max_mhz):
     """FP32-pipe, XU (special-function) and executed-issue fractions of the
-    learned stepper at the measured EM-step rate, from the per-step pipe counts
-    of its ncu capture (profiles/em_kernel_mlp_usr_timed.json, taken at the
-    timed configuration): thread instructions per step on the FMA pipes
-    against SMs x 128 lanes x clock, on the XU against SMs x 16 x clock, and
-    all executed thread instructions against the issue peak."""
+    learned stepper at the measured EM-step rate, from the per-step counts of
+    its ncu capture (profiles/em_kernel_mlp_usr_timed.json: the timed
+    configuration with a quarter of its trajectories): warp instructions x 32
+    per step on the FMA pipes against SMs x 128 lanes x clock, on the XU
+    against SMs x 16 x clock, and all executed thread instructions against the
+    issue peak. The counts are those of the commit that `pipes_source` names."""
     path = os.path.join(ROOT, "profiles", "em_kernel_mlp_usr_timed.json")
     try:
         with open(path) as f:
@@ -202,10 +203,10 @@ def pipe_fractions(steps_per_s, sm_count, sm_max_mhz):
     clk = sm_max_mhz * 1e6
     per = pr.get("per_step", {})
     out = {"pipes_source": f"profiles/em_kernel_mlp_usr_timed.json (ncu, commit {pr.get('commit', '?')})"}
-    if "thread_inst_fma" in per:
-        out["fp32_pipe_frac"] = round(per["thread_inst_fma"] * steps_per_s / (sm_count * SM_LANES * clk), 4)
-    if "thread_inst_xu" in per:
-        out["xu_frac"] = round(per["thread_inst_xu"] * steps_per_s / (sm_count * 16 * clk), 4)
+    if "warp_inst_x32_fma" in per:
+        out["fp32_pipe_frac"] = round(per["warp_inst_x32_fma"] * steps_per_s / (sm_count * SM_LANES * clk), 4)
+    if "warp_inst_x32_xu" in per:
+        out["xu_frac"] = round(per["warp_inst_x32_xu"] * steps_per_s / (sm_count * 16 * clk), 4)
     if "thread_inst" in per:
         out["executed_instr_per_step"] = per["thread_inst"]
         out["issue_frac_executed"] = round(per["thread_inst"] * steps_per_s / (sm_count * SM_LANES * clk), 4)
