@@ -124,8 +124,8 @@ __device__ __forceinline__ float sqrt_approx(float v)
 // 2^-22: neither is ever subnormal, so the flushing forms of the hardware
 // functions give the same bits without their subnormal handling, and -2 ln u0
 // is positive (all of this compared bit for bit over the 2^23 uniforms).
-// Executed instructions per step of direct sampling: 52.5, with the chained passage
-// test 50.8; with the lane's Philox products 38.1 -> 37.2 ms on 2^22 paths, noise
+// Executed instructions per step of direct sampling: 51.0 (52.5 before the chained
+// passage test); with the lane's Philox products 38.1 -> 37.2 ms on 2^22 paths, noise
 // window 26.1 -> 24.6 ms and bump 10.6 -> 10.2 ms on 10^6.
 __device__ __forceinline__ float uniform23(uint32_t r)
 {
@@ -1676,8 +1676,8 @@ __global__ void __launch_bounds__(256) hist_max_kernel(const HistParams P)
         if (s_max[i] && s_max[i] > *(volatile unsigned long long *)&S.key[i]) atomicMax(&S.key[i], s_max[i]);
 }
 
-// exp(d) for d <= 0 (0 below -708, where the result leaves the normal range):
-// d = k ln2/256 + r, |r| < 0.00136, exp(d) = 2^(k >> 8) 2^((k & 255)/256) exp(r)
+// exp(d) for d <= 0 (0 below -708, where the result leaves the normal range), by
+// Tang's table-driven method (ACM TOMS 15, 1989): d = k ln2/256 + r, |r| < 0.00136, exp(d) = 2^(k >> 8) 2^((k & 255)/256) exp(r)
 // with exp(r) to r^4/24 (next term 4e-17) and ln2/256 in two parts.
 __device__ __forceinline__ double exp_neg(double d, const double *__restrict__ tab)
 {
