@@ -389,7 +389,10 @@ fpt_status fpt_histogram(fpt_ctx *ctx, int32_t run, double N_lo, double N_hi,
  * The same weighted histogram over caller-supplied per-trajectory arrays
  * (n entries each, host or device; status as FPT_TRAJ_*), e.g. the merged
  * results of several fpt_run calls. Trajectories are numbered 0..n-1 for the
- * jackknife blocks. Blocks until the results are on the host.
+ * jackknife blocks. ln w may be -inf (weight zero): such a path counts, and has
+ * no share in the weighted sums of its bin or of the scalars; in a bin of
+ * nothing else the logarithms of the sums, pdf and se_jk are NaN. Blocks until
+ * the results are on the host.
  */
 fpt_status fpt_histogram_data(fpt_ctx *ctx, const int32_t *nsteps, const double *logw,
                               const uint8_t *status, int64_t n, double dN, double N_lo,

@@ -1691,7 +1691,7 @@ __device__ __forceinline__ double exp_neg(double d, const double *__restrict__ t
     const double p = fma(r * r, q, r);
     const double T = tab[k & 255];
     const double e = fma(T, p, T);
-    const double s = __hiloint2double(__double2hiint(e) + (k >> 8) * (1 << 20), __double2loint(e));
+    const double s = __hiloint2double(__double2hiint(e) + (int)((unsigned)(k >> 8) << 20), __double2loint(e));
     const unsigned a = (unsigned)__double2hiint(d) & 0x7fffffffu;
     return a > 0x7ff00000u ? d : a > 0x40862000u ? 0.0 : s;      // NaN; |d| > 708
 }
